@@ -1405,11 +1405,248 @@ __device__ void pcgrad_fast(const double* G, uint64_t seed, uint64_t step, int64
 }
 
 // ---------------------------------------------------------------------------
+// K >= 3: the usual support first
+// ---------------------------------------------------------------------------
+//
+// MGDA and CAGrad supports are found here by a few rounds of block pivoting
+// from the full set (languages' gradients of one model mostly all take part):
+// solve on the support, drop what comes out negative, add what violates the
+// optimality condition, until neither happens.  Lane i holds row i of G_SS
+// (rows outside S are unit rows) factored without pivoting in fp32 -- G_SS is
+// positive definite, and a small pivot ends the attempt -- then the solution
+// is refined against the fp64 Gram and certified like every fast path.  What
+// this does not settle goes to the enumeration (K <= 5) or the active-set
+// method below.  Straight-line code of a few KB: a solve runs once per bucket
+// on an SM whose instruction caches hold other code, so its size counts.  One
+// warp alone, cycles: MGDA K = 8 7.5k (about 64k before, by the active-set
+// method, which solves up to K larger systems), CAGrad K = 8 22k (56k).
+// Three launches over a plan of four K = 8 buckets: 74 -> 37 us.
+
+// Sum over the first KM lanes, on every lane.
+template <int KM>
+__device__ __forceinline__ double sum_lanes(double x) {
+#pragma unroll
+  for (int off = KM <= 4 ? 2 : KM <= 8 ? 4 : 8; off > 0; off >>= 1)
+    x += __shfl_xor_sync(0xffffffffu, x, off);
+  return __shfl_sync(0xffffffffu, x, 0);
+}
+template <int KM>
+__device__ __forceinline__ float sum_lanes_f(float x) {
+#pragma unroll
+  for (int off = KM <= 4 ? 2 : KM <= 8 ? 4 : 8; off > 0; off >>= 1)
+    x += __shfl_xor_sync(0xffffffffu, x, off);
+  return __shfl_sync(0xffffffffu, x, 0);
+}
+
+// LU factors of G_SS: multipliers left of the diagonal, reciprocal pivots on
+// it, U right of it.  Returns the smallest pivot.
+template <int KM>
+__device__ __forceinline__ float lu_factor(float (&a)[KM], const float* Gf, int K, unsigned S,
+                                           int lane) {
+  const bool in = (S >> lane) & 1u;
+#pragma unroll
+  for (int j = 0; j < KM; ++j)
+    a[j] = (in && ((S >> j) & 1u)) ? Gf[lane * K + j] : (j == lane ? 1.0f : 0.0f);
+  float least = INFINITY;
+#pragma unroll
+  for (int c = 0; c < KM; ++c) {
+    const float d = __shfl_sync(0xffffffffu, a[c], c);
+    least = d < least ? d : least;
+    const float inv = __frcp_rn(d);
+    const float f = lane > c ? a[c] * inv : 0.0f;
+#pragma unroll
+    for (int j = c + 1; j < KM; ++j) a[j] = fmaf(-f, __shfl_sync(0xffffffffu, a[j], c), a[j]);
+    if (lane > c) a[c] = f;
+    if (lane == c) a[c] = inv;
+  }
+  return least;
+}
+template <int KM>
+__device__ __forceinline__ float lu_solve(const float (&a)[KM], float y, int lane) {
+#pragma unroll
+  for (int c = 0; c + 1 < KM; ++c) {
+    const float yc = __shfl_sync(0xffffffffu, y, c);
+    if (lane > c) y = fmaf(-a[c], yc, y);
+  }
+#pragma unroll
+  for (int c = KM - 1; c >= 0; --c) {
+    if (lane == c) y *= a[c];
+    const float xc = __shfl_sync(0xffffffffu, y, c);
+    if (lane < c) y = fmaf(-a[c], xc, y);
+  }
+  return y;
+}
+// Row `lane` of G times x (lane j holds x_j), fp64 and fp32.
+template <int KM>
+__device__ __forceinline__ double g_times(const double* G, int K, double x, int lane) {
+  double v = 0.0;
+  const int r = (lane < K ? lane : 0) * K;
+#pragma unroll
+  for (int j = 0; j < KM; ++j) {
+    const double xj = __shfl_sync(0xffffffffu, x, j);
+    if (j < K) v = fma(G[r + j], xj, v);
+  }
+  return v;
+}
+template <int KM>
+__device__ __forceinline__ float g_times_f(const float* Gf, int K, float x, int lane) {
+  float v = 0.0f;
+  const int r = (lane < K ? lane : 0) * K;
+#pragma unroll
+  for (int j = 0; j < KM; ++j) {
+    const float xj = __shfl_sync(0xffffffffu, x, j);
+    if (j < K) v = fmaf(Gf[r + j], xj, v);
+  }
+  return v;
+}
+
+constexpr int kPivotRounds = 4;
+constexpr float kLeastPivot = 1e-5f;   // below: not this method (max_k G_kk is in [1, 2))
+constexpr float kEasyPivot = 0.03f;    // above: one refinement reaches fp64 accuracy
+
+// x (G_SS x = rhs on the support) refined against the fp64 Gram.
+template <int KM>
+__device__ __forceinline__ double lu_refine(const float (&a)[KM], const double* G, int K, double x,
+                                            double rhs, bool in, int lane, int steps) {
+#pragma unroll 1
+  for (int i = 0; i < steps; ++i) {
+    const double v = g_times<KM>(G, K, x, lane);
+    x += (double)lu_solve<KM>(a, in ? (float)(rhs - v) : 0.0f, lane);
+  }
+  return x;
+}
+
+template <int KM>
+__device__ bool mgda_pivot(int K, const double* G, const float* Gf, int lane, double* beta_out) {
+  const bool act = lane < K;
+  unsigned S = (1u << K) - 1u;
+  float a[KM], x = 0.0f, least = 0.0f;
+  bool done = false;
+#pragma unroll 1
+  for (int it = 0; it < kPivotRounds && !done; ++it) {
+    least = lu_factor<KM>(a, Gf, K, S, lane);
+    if (!(least > kLeastPivot)) return false;
+    const bool in = (S >> lane) & 1u;
+    x = lu_solve<KM>(a, in ? 1.0f : 0.0f, lane);
+    const float s = sum_lanes_f<KM>(x);
+    if (!(s > 0.0f)) return false;
+    const unsigned neg = __ballot_sync(0xffffffffu, in && !(x > 1e-7f * s));
+    if (neg) {
+      S &= ~neg;
+      if (S == 0u) return false;
+      continue;
+    }
+    // G x >= 1 off the support (its value on it)
+    const float v = g_times_f<KM>(Gf, K, x, lane);
+    const unsigned viol = __ballot_sync(0xffffffffu, act && !in && v < 1.0f - 1e-6f * s);
+    S |= viol;
+    done = viol == 0u;
+  }
+  if (!done) return false;
+  const bool in = (S >> lane) & 1u;
+  const double z = lu_refine<KM>(a, G, K, (double)x, 1.0, in, lane, least > kEasyPivot ? 1 : 3);
+  double alpha = (in && z > 0.0) ? z : 0.0;
+  alpha *= div_nr(1.0, sum_lanes<KM>(alpha));
+  if (!act) alpha = 0.0;
+  // optimality (proof of Theorem 3.1): fp32 with a margin, fp64 if marginal
+  const float a32 = (float)alpha;
+  const float v32 = g_times_f<KM>(Gf, K, a32, lane);
+  const float xx32 = sum_lanes_f<KM>(act ? a32 * v32 : 0.0f);
+  if (!__all_sync(0xffffffffu, !act || in || (v32 - xx32 >= 1e-5f))) {
+    const double v = g_times<KM>(G, K, alpha, lane);
+    const double xx = sum_lanes<KM>(act ? alpha * v : 0.0);
+    if (!__all_sync(0xffffffffu, !act || v >= xx - kKkt)) return false;
+  }
+  if (act) beta_out[lane] = alpha;
+  return true;
+}
+
+template <int KM>
+__device__ bool cagrad_pivot(int K, const double* G, const float* Gf, double c, int lane,
+                             double* beta_out) {
+  const bool act = lane < K;
+  // b_k = <g_k, g0>, ||g0||^2
+  const double ik = div_nr(1.0, (double)K);
+  const double gi = g_times<KM>(G, K, ik, lane);   // (every lane takes part)
+  const double bd = act ? gi : 0.0;
+  const double g0sq = sum_lanes<KM>(bd) * ik;
+  if (!(c > 0.0) || !(g0sq > 0.0)) return false;
+  const double rho = c * sqrt_nr(g0sq);
+  const float rhof = (float)rho, bf = (float)bd;
+  unsigned S = (1u << K) - 1u;
+  float a[KM], m = 0.0f, n = 0.0f, least = 0.0f;
+  bool done = false;
+#pragma unroll 1
+  for (int it = 0; it < kPivotRounds && !done; ++it) {
+    least = lu_factor<KM>(a, Gf, K, S, lane);
+    if (!(least > kLeastPivot)) return false;
+    const bool in = (S >> lane) & 1u;
+    m = lu_solve<KM>(a, in ? 1.0f : 0.0f, lane);
+    n = lu_solve<KM>(a, in ? bf : 0.0f, lane);
+    const float om = sum_lanes_f<KM>(m), on = sum_lanes_f<KM>(n);
+    const float nb = sum_lanes_f<KM>(in ? n * bf : 0.0f);
+    const float D = on * on - om * (nb - rhof * rhof);
+    if (!(om > 0.0f) || !(D > 0.0f)) return false;
+    const float sd = sqrtf(D), lamc = (on + sd) / om;
+    const float w = in ? (lamc * m - n) / sd : 0.0f;
+    const unsigned neg = __ballot_sync(0xffffffffu, in && !(w > 1e-7f));
+    if (neg) {
+      S &= ~neg;
+      if (S == 0u) return false;
+      continue;
+    }
+    const float v = g_times_f<KM>(Gf, K, w, lane);
+    const float q = sum_lanes_f<KM>(in ? w * v : 0.0f);
+    if (!(q > 1e-20f)) return false;
+    const float gk = bf + rhof * v / sqrtf(q);
+    const float lam = sum_lanes_f<KM>(in ? w * gk : 0.0f);
+    const unsigned viol = __ballot_sync(0xffffffffu, act && !in && gk < lam - 1e-6f);
+    S |= viol;
+    done = viol == 0u;
+  }
+  if (!done) return false;
+  const bool in = (S >> lane) & 1u;
+  const int steps = least > kEasyPivot ? 1 : 3;
+  const double md = lu_refine<KM>(a, G, K, in ? (double)m : 0.0, 1.0, in, lane, steps);
+  const double nd = lu_refine<KM>(a, G, K, in ? (double)n : 0.0, bd, in, lane, steps);
+  const double om = sum_lanes<KM>(in ? md : 0.0), on = sum_lanes<KM>(in ? nd : 0.0);
+  const double nb = sum_lanes<KM>(in ? nd * bd : 0.0);
+  const double D = on * on - om * (nb - rho * rho);
+  if (!(om > 0.0) || !(D > 0.0)) return false;
+  const double sd = sqrt_nr(D), lamc = div_nr(on + sd, om), isd = div_nr(1.0, sd);
+  const double zi = in ? (lamc * md - nd) * isd : 0.0;
+  double wd = zi > 0.0 ? zi : 0.0;
+  wd *= (2.0 - sum_lanes<KM>(wd));
+  if (!act) wd = 0.0;
+  // optimality of the dual, and beta = 1/K + rho w / ||g_w|| in fp64
+  const double vd = g_times<KM>(G, K, wd, lane);
+  const double qd = sum_lanes<KM>(act ? wd * vd : 0.0);
+  if (!(qd > 1e-24)) return false;
+  const double f = div_nr(rho, sqrt_nr(qd));
+  const double gk = act ? fma(f, vd, bd) : 1e300;
+  const double lam = sum_lanes<KM>(act ? wd * gk : 0.0);
+  if (!__all_sync(0xffffffffu, !act || in || gk >= lam - 1e-11)) return false;
+  if (act) beta_out[lane] = fma(f, wd, 1.0 / K);
+  return true;
+}
+
+// Rules with a support, K >= 3 (see above).  KM: at least K.
+template <int KM>
+__device__ __noinline__ bool solve_pivot(int K, int rule, const double* G, const float* Gf,
+                                         const SolveParams& p, int lane, double* beta_out) {
+  if (!(p.flags & BKMOO_FLAG_POLISH)) return false;
+  if (rule == BKMOO_MGDA) return mgda_pivot<KM>(K, G, Gf, lane, beta_out);
+  if (rule == BKMOO_CAGRAD) return cagrad_pivot<KM>(K, G, Gf, p.cagrad_c, lane, beta_out);
+  return false;
+}
+
+// ---------------------------------------------------------------------------
 // K >= 6: Wolfe's algorithm in fp32 with a lane-parallel Gauss-Jordan
 // ---------------------------------------------------------------------------
 
-constexpr int kUnk = kMaxK + 1;   // up to kMaxK + 1 unknowns
-constexpr int kCols = kUnk + 2;   // two right-hand sides in slots kUnk, kUnk + 1
+// KM: the largest K a copy serves; a row has unk(KM) = KM + 1 unknowns and two
+// right-hand sides in the slots after them.
+__host__ __device__ constexpr int unk(int KM) { return KM + 1; }
 
 // Position of the n-th (0-based) set bit of m.
 __device__ __forceinline__ int nth_set(unsigned m, int n) {
@@ -1429,7 +1666,9 @@ __device__ __forceinline__ float warp_sum_f(float x) {
 // row[kUnk + 1].  Gauss-Jordan with partial pivoting across lanes;
 // afterwards lane i < m holds the two solutions' i-th entries in the same
 // slots.  False when a pivot is below `piv`.
-__device__ bool warp_gauss_jordan(float (&row)[kCols], int m, int lane, float piv) {
+template <int KM>
+__device__ bool warp_gauss_jordan(float (&row)[unk(KM) + 2], int m, int lane, float piv) {
+  constexpr int kUnk = unk(KM), kCols = kUnk + 2;
   bool ok = true;
 #pragma unroll
   for (int c = 0; c < kUnk; ++c) {
@@ -1445,9 +1684,11 @@ __device__ bool warp_gauss_jordan(float (&row)[kCols], int m, int lane, float pi
       }
     }
     if (!(a > piv)) ok = false;
-    const int src = lane == c ? p : (lane == p ? c : lane);
+    if (p != c) {   // the same on every lane; rare, the diagonal leads
+      const int src = lane == c ? p : (lane == p ? c : lane);
 #pragma unroll
-    for (int j = c; j < kCols; ++j) row[j] = __shfl_sync(0xffffffffu, row[j], src);
+      for (int j = c; j < kCols; ++j) row[j] = __shfl_sync(0xffffffffu, row[j], src);
+    }
     const float inv = __frcp_rn(__shfl_sync(0xffffffffu, row[c], c));
     const float f = row[c];
 #pragma unroll
@@ -1462,8 +1703,10 @@ __device__ bool warp_gauss_jordan(float (&row)[kCols], int m, int lane, float pi
 
 // Bordered system of the affine minimum-norm point of support smask
 // (s = |S| rows of G_SS | 1, then the row 1^T | 0); rhs supplied per lane.
+template <int KM>
 __device__ __forceinline__ void mgda_rows(const float* Gf, int K, unsigned smask, int lane,
-                                          float rhs, float (&row)[kCols]) {
+                                          float rhs, float (&row)[unk(KM) + 2]) {
+  constexpr int kUnk = unk(KM);
   const int s = __popc(smask);
   const int pi = lane < s ? nth_set(smask, lane) : 0;
 #pragma unroll
@@ -1485,13 +1728,16 @@ __device__ __forceinline__ void mgda_rows(const float* Gf, int K, unsigned smask
 // on the fp32 Gram with lane k holding weight lam_k, then one fp64
 // refinement of the final support and the optimality check.  False (beta
 // untouched) if a system is singular or the check fails.
+template <int KM>
 __device__ bool mgda_wolfe_warp(int K, const double* G, const float* Gf, int lane,
                                 double* beta_out) {
+  constexpr int kUnk = unk(KM);
   const bool act = lane < K;
   const int k0 = warp_argmin_f(act ? Gf[lane * K + lane] : INFINITY, lane);
   bool in = lane == k0;
   float lam = in ? 1.0f : 0.0f;
-  float row[kCols];
+  float row[kUnk + 2];
+  unsigned solved = 0;   // the support whose system `row` holds the solution of
   for (int major = 0; major < 4 * K + 4; ++major) {
     float v = 0.0f;
     for (int j = 0; j < K; ++j) {
@@ -1512,8 +1758,9 @@ __device__ bool mgda_wolfe_warp(int K, const double* G, const float* Gf, int lan
       const unsigned smask = __ballot_sync(0xffffffffu, in && act);
       const int s = __popc(smask);
       if (s == 0) return false;
-      mgda_rows(Gf, K, smask, lane, lane == s ? 1.0f : 0.0f, row);
-      if (!warp_gauss_jordan(row, s + 1, lane, 1e-6f)) return false;
+      mgda_rows<KM>(Gf, K, smask, lane, lane == s ? 1.0f : 0.0f, row);
+      if (!warp_gauss_jordan<KM>(row, s + 1, lane, 1e-6f)) return false;
+      solved = smask;
       const int rank = __popc(smask & ((1u << lane) - 1u));
       const float mu_all = __shfl_sync(0xffffffffu, row[kUnk], in ? rank : 0);
       const float mu = in ? mu_all : 0.0f;
@@ -1538,8 +1785,10 @@ __device__ bool mgda_wolfe_warp(int K, const double* G, const float* Gf, int lan
   const unsigned smask = __ballot_sync(0xffffffffu, in && act);
   const int s = __popc(smask);
   if (s == 0) return false;
-  mgda_rows(Gf, K, smask, lane, lane == s ? 1.0f : 0.0f, row);
-  if (!warp_gauss_jordan(row, s + 1, lane, 1e-6f)) return false;
+  if (smask != solved) {
+    mgda_rows<KM>(Gf, K, smask, lane, lane == s ? 1.0f : 0.0f, row);
+    if (!warp_gauss_jordan<KM>(row, s + 1, lane, 1e-6f)) return false;
+  }
   double z = (lane <= s) ? (double)row[kUnk] : 0.0;   // lane i <= s: unknown i
   double r = 0.0;
   {
@@ -1556,8 +1805,8 @@ __device__ bool mgda_wolfe_warp(int K, const double* G, const float* Gf, int lan
     }
     r = lane < s ? -acc : (lane == s ? 1.0 - acc : 0.0);
   }
-  mgda_rows(Gf, K, smask, lane, (float)r, row);
-  if (!warp_gauss_jordan(row, s + 1, lane, 1e-6f)) return false;
+  mgda_rows<KM>(Gf, K, smask, lane, (float)r, row);
+  if (!warp_gauss_jordan<KM>(row, s + 1, lane, 1e-6f)) return false;
   z += (lane <= s) ? (double)row[kUnk] : 0.0;
   // alpha on lanes k < K
   const int rank = __popc(smask & ((1u << lane) - 1u));
@@ -1591,8 +1840,10 @@ __device__ bool mgda_wolfe_warp(int K, const double* G, const float* Gf, int lan
 }
 
 // Rows of G_SS [m n] = [1 b_S] for support smask (lane i < s: row i).
+template <int KM>
 __device__ __forceinline__ void cagrad_rows(const float* Gf, int K, unsigned smask, int lane,
-                                            float bi, float r1, float r2, float (&row)[kCols]) {
+                                            float r1, float r2, float (&row)[unk(KM) + 2]) {
+  constexpr int kUnk = unk(KM);
   const int s = __popc(smask);
   const int pi = lane < s ? nth_set(smask, lane) : 0;
 #pragma unroll
@@ -1600,7 +1851,6 @@ __device__ __forceinline__ void cagrad_rows(const float* Gf, int K, unsigned sma
     row[j] = (j < s && lane < s) ? Gf[pi * K + nth_set(smask, j)] : 0.0f;
   row[kUnk] = lane < s ? r1 : 0.0f;
   row[kUnk + 1] = lane < s ? r2 : 0.0f;
-  (void)bi;
 }
 
 // Exact CAGrad for any K (used for K >= 6): active-set method on the dual
@@ -1608,8 +1858,10 @@ __device__ __forceinline__ void cagrad_rows(const float* Gf, int K, unsigned sma
 // closed-form stationary point of each support (see cag_affine) solved by
 // the lane-parallel Gauss-Jordan in fp32; then m, n refined once in fp64,
 // the closed form in fp64 and the optimality check.  Lane k holds w_k.
+template <int KM>
 __device__ bool cagrad_active_warp(int K, const double* G, const float* Gf, double c, int lane,
                                    double* beta_out) {
+  constexpr int kUnk = unk(KM);
   const bool act = lane < K;
   // b_k = <g_k, g0>, ||g0||^2 (fp64 for the final coefficients)
   double bd = 0.0;
@@ -1631,7 +1883,8 @@ __device__ bool cagrad_active_warp(int K, const double* G, const float* Gf, doub
   const int k0 = warp_argmin_f(Fv, lane);
   bool in = lane == k0;
   float w = in ? 1.0f : 0.0f;
-  float row[kCols];
+  float row[kUnk + 2];
+  unsigned solved = 0;   // the support whose system `row` holds the solutions of
   for (int major = 0; major < 4 * K + 4; ++major) {
     float v = 0.0f;
     for (int j = 0; j < K; ++j) {
@@ -1655,8 +1908,9 @@ __device__ bool cagrad_active_warp(int K, const double* G, const float* Gf, doub
       const int s = __popc(smask);
       if (s == 0) return false;
       const int pi = lane < s ? nth_set(smask, lane) : 0;
-      cagrad_rows(Gf, K, smask, lane, 0.0f, 1.0f, __shfl_sync(0xffffffffu, bf, pi), row);
-      if (!warp_gauss_jordan(row, s, lane, 1e-6f)) return false;
+      cagrad_rows<KM>(Gf, K, smask, lane, 1.0f, __shfl_sync(0xffffffffu, bf, pi), row);
+      if (!warp_gauss_jordan<KM>(row, s, lane, 1e-6f)) return false;
+      solved = smask;
       const float mi = lane < s ? row[kUnk] : 0.0f, ni = lane < s ? row[kUnk + 1] : 0.0f;
       const float bpi = __shfl_sync(0xffffffffu, bf, pi);
       const float om = warp_sum_f(mi), on = warp_sum_f(ni), nb = warp_sum_f(lane < s ? ni * bpi : 0.0f);
@@ -1690,8 +1944,10 @@ __device__ bool cagrad_active_warp(int K, const double* G, const float* Gf, doub
   if (s == 0) return false;
   const int pi = lane < s ? nth_set(smask, lane) : 0;
   const double bpi = __shfl_sync(0xffffffffu, bd, pi);
-  cagrad_rows(Gf, K, smask, lane, 0.0f, 1.0f, (float)bpi, row);
-  if (!warp_gauss_jordan(row, s, lane, 1e-6f)) return false;
+  if (smask != solved) {
+    cagrad_rows<KM>(Gf, K, smask, lane, 1.0f, (float)bpi, row);
+    if (!warp_gauss_jordan<KM>(row, s, lane, 1e-6f)) return false;
+  }
   double md = lane < s ? (double)row[kUnk] : 0.0, nd = lane < s ? (double)row[kUnk + 1] : 0.0;
   double rm = 0.0, rn = 0.0;
   {
@@ -1707,8 +1963,8 @@ __device__ bool cagrad_active_warp(int K, const double* G, const float* Gf, doub
     rm = lane < s ? 1.0 - am : 0.0;
     rn = lane < s ? bpi - an : 0.0;
   }
-  cagrad_rows(Gf, K, smask, lane, 0.0f, (float)rm, (float)rn, row);
-  if (!warp_gauss_jordan(row, s, lane, 1e-6f)) return false;
+  cagrad_rows<KM>(Gf, K, smask, lane, (float)rm, (float)rn, row);
+  if (!warp_gauss_jordan<KM>(row, s, lane, 1e-6f)) return false;
   if (lane < s) {
     md += (double)row[kUnk];
     nd += (double)row[kUnk + 1];
@@ -1749,27 +2005,36 @@ __device__ bool cagrad_active_warp(int K, const double* G, const float* Gf, doub
   return true;
 }
 
-// Large-K (K > kEnumMaxK) MGDA and CAGrad: one copy of the lane-parallel
-// active-set solvers per kernel, whatever the number of K cases around it.
-__device__ bool solve_large(int K, int rule, const double* G, const float* Gf,
-                            const SolveParams& p, int lane, double* beta_out) {
+// Large-K (K > kEnumMaxK) MGDA and CAGrad by the lane-parallel active-set
+// solvers, from the best vertex.  A copy for K <= KM keeps KM + 1 unknowns
+// per row.
+template <int KM>
+__device__ bool solve_large_k(int K, int rule, const double* G, const float* Gf,
+                              const SolveParams& p, int lane, double* beta_out) {
   if (!(p.flags & BKMOO_FLAG_POLISH)) return false;
-  if (rule == BKMOO_MGDA) return mgda_wolfe_warp(K, G, Gf, lane, beta_out);
-  if (rule == BKMOO_CAGRAD) return cagrad_active_warp(K, G, Gf, p.cagrad_c, lane, beta_out);
+  if (rule == BKMOO_MGDA) return mgda_wolfe_warp<KM>(K, G, Gf, lane, beta_out);
+  if (rule == BKMOO_CAGRAD) return cagrad_active_warp<KM>(K, G, Gf, p.cagrad_c, lane, beta_out);
   return false;
 }
+// K a runtime value: two copies, whatever the number of K cases around it.
+__device__ bool solve_large(int K, int rule, const double* G, const float* Gf,
+                            const SolveParams& p, int lane, double* beta_out) {
+  return K <= 8 ? solve_large_k<8>(K, rule, G, Gf, p, lane, beta_out)
+                : solve_large_k<kMaxK>(K, rule, G, Gf, p, lane, beta_out);
+}
 
+// The support by enumeration (K <= kEnumMaxK) or the active-set method.
 // kLarge: whether this instantiation carries the large-K solvers itself
 // (the runtime-K dispatch below calls solve_large once, outside its switch).
+// Out of line: after solve_pivot it is rarely needed.
 template <int K, bool kLarge>
-__device__ bool solve_fast_k(int rule, const double* G, const float* Gf, const SolveParams& p,
-                             int64_t b, int lane, double* beta_out) {
-  if (rule == BKMOO_PCGRAD) {
-    pcgrad_fast<K>(G, p.seed, p.step, b, lane, beta_out);
-    return true;
+__device__ __noinline__ bool solve_support(int rule, const double* G, const float* Gf,
+                                           const SolveParams& p, int lane, double* beta_out) {
+  if (K > kEnumMaxK) {
+    if constexpr (kLarge && K > kEnumMaxK)
+      return solve_large_k<K>(K, rule, G, Gf, p, lane, beta_out);
+    return false;
   }
-  if (!(p.flags & BKMOO_FLAG_POLISH)) return false;
-  if (K > kEnumMaxK) return kLarge ? solve_large(K, rule, G, Gf, p, lane, beta_out) : false;
   if (rule == BKMOO_MGDA) {
     if (K < 2 || (K == 2 && (p.flags & BKMOO_FLAG_CLOSED_FORM_K2))) return false;
     return mgda_fast<(K <= kEnumMaxK ? K : 2)>(G, Gf, lane, beta_out);
@@ -1784,10 +2049,29 @@ __device__ bool solve_fast_k(int rule, const double* G, const float* Gf, const S
   return false;
 }
 
+template <int K, bool kLarge>
+__device__ __forceinline__ bool solve_fast_k(int rule, const double* G, const float* Gf,
+                                             const SolveParams& p, int64_t b, int lane,
+                                             double* beta_out) {
+  if (rule == BKMOO_PCGRAD) {
+    pcgrad_fast<K>(G, p.seed, p.step, b, lane, beta_out);
+    return true;
+  }
+  if (!(p.flags & BKMOO_FLAG_POLISH) || rule == BKMOO_MEAN) return false;
+  if constexpr (kLarge && K >= 3) {   // (the runtime-K dispatch has tried it)
+    if (solve_pivot<K>(K, rule, G, Gf, p, lane, beta_out)) return true;
+  }
+  return solve_support<K, kLarge>(rule, G, Gf, p, lane, beta_out);
+}
+
 // Dispatch on K; true when a fast path produced beta (valid on every lane
 // after the caller's __syncwarp).
 __device__ bool solve_fast(int K, int rule, const double* G, const float* Gf,
                            const SolveParams& p, int64_t b, int lane, double* beta_out) {
+  if (K >= 3 && (K <= 4   ? solve_pivot<4>(K, rule, G, Gf, p, lane, beta_out)
+                 : K <= 8 ? solve_pivot<8>(K, rule, G, Gf, p, lane, beta_out)
+                          : solve_pivot<kMaxK>(K, rule, G, Gf, p, lane, beta_out)))
+    return true;
   if (K > kEnumMaxK && rule != BKMOO_PCGRAD) return solve_large(K, rule, G, Gf, p, lane, beta_out);
   switch (K) {
 #define BKMOO_FAST_CASE(k) \
@@ -1804,6 +2088,23 @@ __device__ bool solve_fast(int K, int rule, const double* G, const float* Gf,
 // ---------------------------------------------------------------------------
 // per bucket (whole warp)
 // ---------------------------------------------------------------------------
+
+// One lane: the general solvers (Frank-Wolfe with completion, the K = 2 closed
+// form, literal PCGrad, the mean).
+__device__ __noinline__ int solve_lane(int K, const double* G, const SolveParams& q, int64_t b,
+                                       double* beta_out) {
+  double beta[kMaxK];
+  int st = BKMOO_OK;
+  switch (q.rule) {
+    case BKMOO_MGDA: st = solve_mgda(K, G, q, beta); break;
+    case BKMOO_PCGRAD: st = solve_pcgrad(K, G, q, b, beta); break;
+    case BKMOO_CAGRAD: st = solve_cagrad(K, G, q, beta); break;
+    default:
+      for (int k = 0; k < K; ++k) beta[k] = 1.0 / K;
+  }
+  for (int k = 0; k < K; ++k) beta_out[k] = beta[k];
+  return st;
+}
 
 // The whole warp enters with G (K x K) in shared memory; G is normalised in
 // place.  beta_out (shared, K entries) and the returned status are valid on
@@ -1857,17 +2158,7 @@ __device__ int solve_bucket_warp(int K, double* G, float* Gf, const SolveParams&
     fast = solve_fast_k<KC, true>(q.rule, G, Gf, q, b, lane, beta_out);
   else
     fast = solve_fast(K, q.rule, G, Gf, q, b, lane, beta_out);
-  if (!fast && lane == 0) {
-    double beta[kMaxK];
-    switch (q.rule) {
-      case BKMOO_MGDA: st = solve_mgda(K, G, q, beta); break;
-      case BKMOO_PCGRAD: st = solve_pcgrad(K, G, q, b, beta); break;
-      case BKMOO_CAGRAD: st = solve_cagrad(K, G, q, beta); break;
-      default:
-        for (int k = 0; k < K; ++k) beta[k] = 1.0 / K;
-    }
-    for (int k = 0; k < K; ++k) beta_out[k] = beta[k];
-  }
+  if (!fast && lane == 0) st = solve_lane(K, G, q, b, beta_out);
   st = __shfl_sync(0xffffffffu, st, 0);
   __syncwarp();
   return st;
