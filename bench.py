@@ -176,7 +176,7 @@ class ClockSampler:
 
 
 def launches_per_step(w, off, fused):
-    """Kernels of this library one resolve launches: the fused kernel; or
+    """Kernels of this library one resolve launches: the streamed kernel; or
     Gram pass, solve and combination, plus the group pre-reduction of the
     chunk partials when a bucket has more than 1024 chunks."""
     import numpy as np
@@ -458,9 +458,6 @@ def main():
         params.flags |= bk.BKMOO_FLAG_FUSED
     elif a.path == "3pass":
         params.flags |= bk.BKMOO_FLAG_THREE_PASS
-    path_id = bk.bkmoo_resolve_path(w.K, bk.BKMOO_F32 if tdt == torch.float32 else bk.BKMOO_BF16,
-                                    a.rule, off, params.flags)
-    fused = path_id != 0
 
     def step(evs=None):
         if evs is not None:
@@ -507,7 +504,10 @@ def main():
     peak, peak_kind = _peaks()
     e_in = w.elem_bytes
     e_out = out.element_size()
-    if fused:   # one launch: Gram + solve + combination, re-read from L2
+    # one launch records the last three events together after it; a solve and
+    # a combination of their own take microseconds
+    fused = float(per[:, 1:].sum(axis=1).mean()) < 0.005
+    if fused:   # one launch: Gram + solve + combination
         kern = {"fused": (per[:, 0].mean(), (w.K * e_in + e_out) * N, "fused")}
         dom = "fused"
     else:
@@ -539,11 +539,8 @@ def main():
                            "inputs (%.3f GB) fit in L2 and are not flushed: L2-resident "
                            "timing" % (grad_bytes / GB)),
                        parallelism="replicas" if world > 1 else "1 GPU",
-                       path=({1: "fused: one launch, a thread-block cluster per bucket, "
-                                    "combination re-reads each bucket from L2",
-                              2: "fused: one persistent launch, groups of CTAs per bucket, "
-                                 "combination re-reads each bucket from L2"}.get(
-                                  path_id, "gram -> solve -> combine (3 launches)")
+                       path=(("one streamed launch, the combination behind the Gram"
+                              if fused else "gram -> solve -> combine (3 launches)")
                              + (" (chosen per plan)" if a.path == "auto" else ""))),
         "roofline": roofline,
         "step_roofline": {"bytes_2k1": step_bytes_2k1, "bytes_k1": step_bytes_k1,

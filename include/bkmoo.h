@@ -73,57 +73,34 @@ typedef enum { BKMOO_F32 = 0, BKMOO_BF16 = 1 } bkmoo_dtype;
 #define BKMOO_FLAG_POLISH 0x2u         /* exact active-set completion after
                                           the Frank-Wolfe phase (MGDA and
                                           CAGrad)                            */
-#define BKMOO_FLAG_FUSED 0x4u          /* one launch that resolves bucket
-                                          after bucket while the bucket is
-                                          still in L2: a thread-block cluster
-                                          per bucket for K <= 4, groups of
-                                          CTAs for K = 5..8; above, ignored
-                                          (three passes).  On a GB300 the
-                                          cluster kernel is faster than three
-                                          passes for K = 2..4 with buckets of
-                                          2-6 MiB (the per-plan choice takes
-                                          it there, see bkmoo_resolve_path),
-                                          slower for 1 MiB buckets, large
-                                          buckets and K = 1 or 8.  The
-                                          cluster kernel's look-ahead into
-                                          the next bucket can be overridden
-                                          with the environment variable
-                                          BKMOO_CLUSTER_HEAD (items per
-                                          thread).  Results agree
-                                          with the three-pass path to
-                                          rounding, not bit for bit.  The
-                                          groups kernel's L2 budget and
-                                          look-ahead can be overridden with
-                                          the environment variables
-                                          BKMOO_FUSED_L2_BUDGET (bytes) and
-                                          BKMOO_FUSED_LOOKAHEAD (buckets).   */
+#define BKMOO_FLAG_FUSED 0x4u          /* one launch in which the combination
+                                          follows the Gram bucket by bucket
+                                          while the gradients are still on
+                                          the chip, for K <= 8; above, ignored
+                                          (three launches).  The results are
+                                          those of the three launches, bit for
+                                          bit.  Without this flag the faster
+                                          of the two is taken.              */
 #define BKMOO_FLAG_THREE_PASS 0x8u     /* always the three-launch path (Gram,
-                                          solve, combination); without it and
-                                          without BKMOO_FLAG_FUSED the path is
-                                          chosen per plan, see
-                                          bkmoo_resolve_path                 */
-#define BKMOO_FLAG_TEST_WITHHOLD 0x100u /* testing failure detection, with
-                                          BKMOO_FLAG_FUSED only (it selects
-                                          the grid-synchronised fused
-                                          kernel): that kernel never
-                                          publishes bucket 0's
+                                          solve, combination)               */
+#define BKMOO_FLAG_TEST_WITHHOLD 0x100u /* testing failure detection, where
+                                          the one launch runs: it never
+                                          publishes its first bucket's
                                           coefficients, so its bounded waits
-                                          (about 1 s) run out and the call
+                                          (about 2 s) run out and the call
                                           ends with BKMOO_ERR_TIMEOUT in the
                                           workspace status word; the output
                                           is then undefined                 */
 #define BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE 0x200u /* testing failure detection,
-                                          with BKMOO_FLAG_FUSED and K <= 4
-                                          only (the cluster kernel): CTA 0
-                                          of every cluster never hands its
-                                          partial Gram of the cluster's
-                                          first bucket to its peers, so the
-                                          peers' bounded exchange waits
-                                          (about 1 s) run out, every later
-                                          wait gives up at once, and the
-                                          call ends with BKMOO_ERR_TIMEOUT
-                                          in the workspace status word; the
-                                          output is then undefined          */
+                                          where the one launch runs: its first
+                                          CTA never publishes its first
+                                          chunk's partial Gram, so the bounded
+                                          wait for it (about 2 s) runs out,
+                                          every other wait ends at once, and
+                                          the call ends with
+                                          BKMOO_ERR_TIMEOUT in the workspace
+                                          status word; the output is then
+                                          undefined                         */
 
 typedef struct {
   int32_t max_iter; /* Frank-Wolfe iterations per bucket (MGDA, CAGrad)     */
@@ -135,8 +112,8 @@ typedef struct {
   void* events;     /* tracing: NULL, or an array of 4 cudaEvent_t that
                        bkmoo_resolve records on `stream` before the Gram pass,
                        after it, after the solve and after the combination
-                       (one persistent launch: the middle two are recorded
-                       together after it).  Owned by the caller.           */
+                       (one launch: the last three are recorded together
+                       after it).  Owned by the caller.                    */
 } bkmoo_params;
 
 /* Fill *p with the defaults: max_iter 256, tol 1e-12, cagrad_c 0.5, seed 0,
@@ -287,9 +264,11 @@ int bkmoo_gram_noalloc(const void* const* grads, int32_t K, int32_t in_dtype,
  *   BKMOO_ERR_WORKSPACE; or NULL.
  * ws / ws_bytes: the workspace after bkmoo_workspace_init with the same
  *   K, in_dtype and offsets.
- * Path: three launches (Gram, solve, combination) or one fused launch, as
- *   bkmoo_resolve_path gives for the plan, rule and p->flags.  Each path is
- *   deterministic; the two agree to rounding.
+ * Path: three launches (Gram, solve, combination) or one launch that does the
+ *   same bucket by bucket (see BKMOO_FLAG_FUSED), whichever is faster for the
+ *   plan and rule; the results are the same bit for bit and deterministic.
+ *   The one launch is cooperative (every CTA resident at once); on a device
+ *   or context that cannot hold it the three launches run.
  * Returns BKMOO_OK once the work is queued on `stream`.
  */
 int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype,
@@ -311,8 +290,8 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype,
  * elements of out_dir, the rows of out_weights / out_status and the
  * workspace partials of other buckets are not touched, so calls for disjoint
  * bucket ranges may run concurrently on different streams.  Results are
- * bit-identical to those of bkmoo_resolve's three-launch path for the same
- * buckets.  The workspace
+ * bit-identical to those of bkmoo_resolve for the same buckets; the path is
+ * chosen as there.  The workspace
  * status word is not cleared (other calls may be in flight); device-side
  * errors are recorded into it.  BKMOO_FLAG_FUSED and p->events are ignored.
  */
@@ -380,21 +359,20 @@ int bkmoo_resolve_host(const void* const* host_grads, int32_t K, int32_t in_dtyp
 int bkmoo_workspace_status(const void* ws, void* stream, int32_t* status);
 
 /*
- * bkmoo_resolve_path -- which path bkmoo_resolve takes for this plan, rule
- * and flags: *path = 0 for the three launches (Gram, solve, combination), 1
- * for the cluster-per-bucket fused kernel (one bucket per thread-block
- * cluster, its re-read served from L2), 2 for the grid-synchronised fused
- * kernel.  BKMOO_FLAG_THREE_PASS gives 0; BKMOO_FLAG_FUSED gives 1 for
- * K <= 4 (2 with BKMOO_FLAG_TEST_WITHHOLD), 2 for K = 5..8, 0 above.
- * Without either flag the choice follows measurements on GB300 (sweeps of
- * 1e9 elements per language, fp32 and bf16, and small plans): 1 when K <= 2
- * and the plan has at most 8 buckets and 4 Mi elements per language (one
- * launch instead of three), or when 2 <= K <= 4, the largest bucket holds at
- * least 2 MiB per language and its K gradients together at most 12 MiB
- * (and at least 6 MiB for bf16; for CAGrad, whose per-bucket solve is
- * longer, fp32 only and at least 8 MiB), and at least 90 % of the
- * elements lie in buckets of at least half the largest; 0 otherwise.  Host only; BKMOO_ERR_INVALID on bad arguments.
- * bkmoo_resolve_buckets and bkmoo_resolve_host always take path 0.
+ * bkmoo_resolve_path -- what is certain of bkmoo_resolve's path for this
+ * plan, rule and flags: *path = 1 or 2 for one launch (see BKMOO_FLAG_FUSED),
+ * 0 where it may take the three launches.  (1 and 2 named two earlier one-launch
+ * kernels and keep their conditions; the same kernel now runs for both.)
+ * BKMOO_FLAG_THREE_PASS gives 0 (always three launches); BKMOO_FLAG_FUSED
+ * gives 1 for K <= 4 (2 with BKMOO_FLAG_TEST_WITHHOLD), 2 for K = 5..8, 0
+ * above.  Without either flag: 1 when K <= 2 and the plan has at most 8
+ * buckets and 4 Mi elements per language, or when 2 <= K <= 4, the largest
+ * bucket holds at least 2 MiB per language and its K gradients together at
+ * most 12 MiB (and at least 6 MiB for bf16; for CAGrad fp32 only and at least
+ * 8 MiB), and at least 90 % of the elements lie in buckets of at least half
+ * the largest; 0 otherwise, where one launch runs for most plans of K <= 4 and
+ * many of K = 5..8.  Host only; BKMOO_ERR_INVALID on bad arguments.
+ * bkmoo_resolve_host always takes the three launches per window.
  */
 int bkmoo_resolve_path(int32_t K, int32_t in_dtype, int32_t rule, const int64_t* offsets,
                        int64_t n_buckets, uint32_t flags, int32_t* path);

@@ -12,37 +12,22 @@
 namespace bkmoo {
 
 constexpr int kMaxK = 16;
-// Largest K the fused persistent kernel is built for: above it the per-thread
-// streaming state (K(K+1)/2 accumulators, K vectors in flight) no longer fits
-// the register file, and the three-pass path runs instead.
-constexpr int kFusedMaxK = 8;
+// Largest K of the streamed kernel (stream_resolve.cuh).
+constexpr int kStreamMaxK = 8;
 constexpr int kThreads = 256;              // CTA size of the streaming kernels
 constexpr int kWarps = kThreads / 32;
 constexpr int kVecPerThread = 16;          // 16-byte vectors per thread per Gram chunk
 constexpr uint32_t kMagic = 0x4f4d4b42u;   // "BKMO"
 constexpr int kSolveWarpsPerBlock = 4;
-constexpr int kFusedMaxCtas = 2048;        // upper bound of the fused grid
-// Fused kernel: 11 streaming warps and one solver warp per CTA (12 warps:
-// registers are allocated to warps in groups of four, so 9 warps would cost
-// as many registers as 12); each group of CTAs keeps the CTA partials of its
-// last kFusedRing buckets in a ring.
-constexpr int kFusedStreamWarps = 11;
-constexpr int kFusedThreads = 32 * (kFusedStreamWarps + 1);
-constexpr int kFusedRing = 4;
-// cp.async stages per streaming lane of the fused kernel: about 14 K-vector
-// sets in flight per lane (~80 KB per SM with 11 streaming warps).
-__host__ __device__ constexpr int fused_stages(int K) {
-  return K <= 1 ? 12 : K == 2 ? 8 : K == 3 ? 6 : K == 4 ? 5 : K <= 6 ? 4 : 3;
-}
-__host__ __device__ constexpr int fused_smem_bytes(int K) {
-  return fused_stages(K) * K * 16 * 32 * kFusedStreamWarps;
-}
 // A bucket with more than kGroupMinChunks chunks has its chunk partials
 // pre-reduced in groups of kGroupChunks (group_reduce_kernel, solve.cu)
 // before the per-bucket reduction reads them: one warp would otherwise read
 // every partial of a huge bucket (the one-bucket "global" variant) alone.
 constexpr int64_t kGroupChunks = 512;
 constexpr int64_t kGroupMinChunks = 1024;
+
+// Chunk rows are summed in sets of kSetChunks (K <= kStreamMaxK).
+constexpr int kSetChunks = 16;
 
 __host__ __device__ constexpr int tri(int K) { return K * (K + 1) / 2; }
 __host__ __device__ constexpr int elems_per_vec(int dtype) { return dtype == BKMOO_F32 ? 4 : 8; }
@@ -72,12 +57,10 @@ struct WsLayout {
   size_t partials;       // double [n_chunks][P] per-chunk Gram partials
   size_t beta;           // float [B][K]    coefficients of the last resolve
   size_t total;          // end of the regions above
-  // fused path only (bkmoo_resolve with BKMOO_FLAG_FUSED):
-  size_t arrive;         // int32 [B]      CTAs of bucket b's group done with its Gram
-  size_t ready;          // int32 [B + 1]  1 once beta of bucket b is written;
-                         //                [B] counts the buckets published
-  size_t ring;           // double [kFusedRing][2 kFusedMaxCtas][P] CTA partials
-  size_t total_fused;
+  // streamed path only
+  size_t rows;           // uint64 [n_chunks][stream_row_words(K)], K <= kStreamMaxK
+  size_t chunk_bucket;   // int32 [n_chunks] bucket of each chunk
+  size_t total_all;
 };
 
 __host__ __device__ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -126,13 +109,12 @@ __host__ __device__ inline WsLayout ws_layout(int K, int64_t B, int64_t n_chunks
   L.beta = at;
   at = align256(at + sizeof(float) * (size_t)B * (size_t)K);
   L.total = at;
-  L.arrive = at;
-  at = align256(at + sizeof(int32_t) * (size_t)B);
-  L.ready = at;
-  at = align256(at + sizeof(int32_t) * (size_t)(B + 1));
-  L.ring = at;
-  at = align256(at + sizeof(double) * kFusedRing * 2 * (size_t)kFusedMaxCtas * (size_t)tri(K));
-  L.total_fused = at;
+  L.rows = at;
+  if (K <= kStreamMaxK)
+    at = align256(at + sizeof(uint64_t) * (size_t)n_chunks * (size_t)(tri(K) + K + 1));
+  L.chunk_bucket = at;
+  at = align256(at + sizeof(int32_t) * (size_t)n_chunks);
+  L.total_all = at;
   return L;
 }
 
@@ -168,19 +150,26 @@ __host__ __device__ inline void full_window(PlanView& v) {
   v.b_hi = v.n_buckets;
 }
 
-// The fused path's view: the plan plus the synchronisation arrays.  CTA c
-// belongs to group c % n_groups; bucket b is resolved by group b % n_groups.
-struct FusedView {
+// The streamed path's view (stream_resolve.cuh): the plan's window plus one
+// row of 64-bit words per chunk:
+//   [0, P)       the chunk's partials,
+//   [P, P + K)   in a bucket's first chunk: the bucket's coefficients,
+//   [P + K]      in the window's first row: the give-up flag.
+// Every word is 0 until it is written (see st_row and st_beta).
+struct StreamView {
   PlanView v;
-  int32_t* arrive;
-  int32_t* ready;
-  double* ring;          // [n_groups][kFusedRing][group_ctas][P]
-  float* out_weights;
-  int32_t* out_status;
-  int32_t n_groups;
-  int32_t group_ctas;    // rows of a ring slot: CTAs of the largest group
-  int32_t lookahead;     // buckets a warp's Gram may run ahead of its combination
+  uint64_t* rows;               // row of chunk w0
+  const int32_t* chunk_bucket;  // bucket of every chunk of the plan
+  int32_t* give_up;             // set once a wait for another CTA ran out
+  int64_t w0;                   // first chunk of the window
+  int32_t lead;                 // stages the Gram may run ahead of the combination
+  int32_t l2_stages;            // stages a CTA asks L2 to keep
+  int32_t n_stream;             // CTAs that stream (chunk w0 + i by CTA i mod n_stream); the
+                                // others solve
+  int32_t team;                 // warps of a solver CTA that share a bucket: 2, 4 or 8
+  int32_t reset;                // clear the workspace status word first
 };
+__host__ __device__ constexpr int stream_row_words(int K) { return tri(K) + K + 1; }
 
 struct SolveParams {
   int32_t rule;
@@ -205,6 +194,51 @@ __device__ __forceinline__ bool header_ok(const PlanView& v) {
 
 __device__ __forceinline__ void record_error(WsHeader* h, int code) {
   atomicCAS(&h->status, 0, code);
+}
+
+// Fixed order of the fp64 sums over Gram rows, one entry per thread (rows
+// rs doubles apart): eight interleaved sums (row c into sum c mod 8), then a
+// fixed tree.
+__device__ __forceinline__ double tree8(const double (&t)[8]) {
+  return ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+}
+__device__ __forceinline__ double sum_rows8(const double* src, int64_t rs, int64_t n) {
+  double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  int64_t c = 0;
+  for (; c + 8 <= n; c += 8, src += 8 * rs) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) t[j] += src[j * rs];
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (c + j < n) t[j] += src[j * rs];
+  return tree8(t);
+}
+// A set: the first kSetChunks (or all left) of `left` rows, a whole one in
+// one round trip.
+__device__ __forceinline__ double set_sum(const double* row, int64_t rs, int64_t left) {
+  if (left < kSetChunks) return sum_rows8(row, rs, left);
+  double x[kSetChunks], u[8];
+#pragma unroll
+  for (int i = 0; i < kSetChunks; ++i) x[i] = row[i * rs];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) u[i] = (0.0 + x[i]) + x[i + 8];
+  return tree8(u);
+}
+// Chunk rows: for K <= kStreamMaxK sets of kSetChunks rows, then the sets'
+// sums in the same way -- the order in which the streamed kernel, whose sets
+// are summed by different CTAs, arrives at them.
+__device__ __forceinline__ double sum_chunk_rows(const double* src, int64_t rs, int64_t n, int K) {
+  if (K > kStreamMaxK) return sum_rows8(src, rs, n);
+  double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  for (int64_t c = 0; c < n; c += 8 * kSetChunks) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int64_t at = c + j * kSetChunks;
+      if (at < n) t[j] += set_sum(src + at * rs, rs, n - at);
+    }
+  }
+  return tree8(t);
 }
 
 // Bucket b with chunk_prefix[b] <= w < chunk_prefix[b+1]; `hint` is tried
@@ -297,26 +331,17 @@ int combine_prefetch_smem(int K);
 const void* combine_fn_f32(int K, int dtype_out);
 const void* combine_fn_bf16(int K, int dtype_out);
 
-// Fused kernels, signature (GradPtrs, FusedView, SolveParams, void* out); fused_*.cu.
-const void* fused_fn_f32_k1_4(int K, int dtype_out);
-const void* fused_fn_f32_k5_6(int K, int dtype_out);
-const void* fused_fn_f32_k7_8(int K, int dtype_out);
-const void* fused_fn_bf16_k1_4(int K, int dtype_out);
-const void* fused_fn_bf16_k5_6(int K, int dtype_out);
-const void* fused_fn_bf16_k7_8(int K, int dtype_out);
-
-// Cluster-per-bucket fused kernels (fused_cluster.cu), K <= kClusterMaxK,
-// signature (GradPtrs, PlanView, SolveParams, float* out_weights,
-// int32_t* out_status, void* out, int head), clusters of kClusterCtas CTAs
-// of kClusterThreads threads (15 streaming warps and one solver warp) with
-// fused_cluster_smem(K) bytes of dynamic shared memory.
-constexpr int kClusterMaxK = 4;
-constexpr int kClusterCtas = 8;
-constexpr int kClusterStreamWarps = 15;
-constexpr int kClusterStreamThreads = 32 * kClusterStreamWarps;
-constexpr int kClusterThreads = kClusterStreamThreads + 32;
-const void* fused_cluster_fn(int K, int dti, int dto);
-int fused_cluster_smem(int K);
+// Streamed resolve kernels (stream_*.cu), K <= kStreamMaxK, signature
+// (GradPtrs, StreamView, SolveParams, float* out_weights, int32_t* out_status,
+// void* out, int dtype_out), stream_threads() threads and stream_smem(K) bytes
+// of dynamic shared memory, one CTA per SM, co-resident.
+const void* stream_fn_k1_2(int K, int dti);
+const void* stream_fn_k3_4(int K, int dti);
+const void* stream_fn_k5_6(int K, int dti);
+const void* stream_fn_k7_8(int K, int dti);
+int stream_threads();
+int stream_smem(int K);
+int stream_stage_kib(int K);
 
 // solve.cu
 cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_weights,

@@ -1,12 +1,11 @@
 // Host side of the C ABI (include/bkmoo.h): argument checks, the bucket plan,
 // the workspace image, the launch sequence Gram -> solve -> combine on the
 // caller's stream (whole plan, a bucket range, or windows of buckets staged
-// from host memory), and the fused persistent launch.  Nothing here
+// from host memory), and the streamed launch.  Nothing here
 // allocates device memory (the host path creates two copy streams and a few
 // events per call).
 #include <cuda_runtime.h>
 
-#include <cstdlib>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -73,183 +72,134 @@ const void* gram_fn(int K, int dt) {
 const void* combine_fn(int K, int dti, int dto) {
   return dti == BKMOO_F32 ? combine_fn_f32(K, dto) : combine_fn_bf16(K, dto);
 }
-const void* fused_fn(int K, int dti, int dto) {
-  if (dti == BKMOO_F32)
-    return K <= 4 ? fused_fn_f32_k1_4(K, dto)
-                  : (K <= 6 ? fused_fn_f32_k5_6(K, dto) : fused_fn_f32_k7_8(K, dto));
-  return K <= 4 ? fused_fn_bf16_k1_4(K, dto)
-                : (K <= 6 ? fused_fn_bf16_k5_6(K, dto) : fused_fn_bf16_k7_8(K, dto));
+const void* stream_fn(int K, int dt) {
+  return K <= 2 ? stream_fn_k1_2(K, dt)
+                : (K <= 4 ? stream_fn_k3_4(K, dt)
+                          : (K <= 6 ? stream_fn_k5_6(K, dt) : stream_fn_k7_8(K, dt)));
 }
 
-// Fused-path sizing.  The bytes that pass through L2 between a bucket's Gram
-// read and its re-read are about (lookahead + 1) buckets per group, so the
-// group count is the budget over that (at least 1, at most one group per 4
-// CTAs and one per bucket).  The budget is a fraction of L2 (3/4: measured
-// re-reads of more than about 76 MB of 126 MB fall to HBM speed on this
-// part, but a lookahead of one bucket and this budget measured fastest).
-// BKMOO_FUSED_L2_BUDGET (bytes) and BKMOO_FUSED_LOOKAHEAD (buckets) override
-// the defaults.
-struct FusedShape {
-  int n_groups;
-  int lookahead;
+// Whether the streamed launch is the faster one for a window (both give the
+// same results).  Measured on GB300 against the three launches, K = 2, 4, 5
+// and 8, fp32 and bf16, MGDA, PCGrad and CAGrad, 2^18 to 2^28 elements in
+// buckets of 64 KiB to 100 MiB: it reads the gradients little more than once
+// and is 1.05-2.6 times as fast wherever the SMs' time goes into streaming.
+// It loses where it goes into solves, which it does on the few SMs it sets
+// aside: many buckets of less than 512 KiB of gradients (K = 4 CAGrad, 256
+// buckets of 64 KiB fp32: 61 us against 41), and for K >= 5, whose solves take
+// 10-20 us, small plans (K = 8, 4 Mi bf16 elements: 53 against 50) and buckets
+// under 1 MiB of gradients (K = 8 CAGrad, 2048 of 512 KiB: 409 against 425 us,
+// PCGrad 470 against 444), and with many buckets of which little stays on the
+// chip (K = 8, 134 buckets of 25 MiB bf16: 6.05 ms against 5.95).
+bool stream_wins(const PlanView& v, const int64_t* off) {
+  if (v.K > kStreamMaxK || v.c_hi <= v.c_lo) return false;
+  const int64_t nb = v.b_hi - v.b_lo;
+  const double bytes = (double)(off[v.b_hi] - off[v.b_lo]) * v.K * elem_bytes(v.in_dtype);
+  const double mib = 1024.0 * 1024.0;
+  if (v.K >= 5)
+    return bytes >= 96.0 * mib && bytes >= 1.0 * mib * nb && (nb <= 8 || bytes < 128.0 * mib * nb);
+  return nb <= 64 || bytes >= 0.5 * mib * nb;
+}
+
+// How a window is spread over the SMs, and how far the Gram may run ahead of
+// the combination.
+struct StreamShape {
+  int n_stream, n_solve, team, lead_kib;
 };
-FusedShape fused_shape(int grid, int64_t n_buckets, double bucket_bytes, int l2_bytes) {
-  double budget = 0.75 * (double)l2_bytes;
-  int lookahead = 1;
-  if (const char* e = std::getenv("BKMOO_FUSED_L2_BUDGET")) {
-    const double x = std::atof(e);
-    if (x > 0) budget = x;
-  }
-  if (const char* e = std::getenv("BKMOO_FUSED_LOOKAHEAD")) {
-    const int x = std::atoi(e);
-    if (x >= 0 && x <= kFusedRing - 2) lookahead = x;
-  }
-  double ng = budget / ((lookahead + 1) * (bucket_bytes > 1.0 ? bucket_bytes : 1.0));
-  int64_t n = (int64_t)ng;
-  const int64_t cap = grid / 4 > 0 ? grid / 4 : 1;
-  if (n > cap) n = cap;
-  if (n > n_buckets) n = n_buckets;
-  if (n < 1) n = 1;
-  return FusedShape{(int)n, lookahead};
+StreamShape stream_shape(const PlanView& v, int rule, int sms) {
+  // From a bucket's last partial to its coefficients on every SM, measured
+  // under load (us; globaltimer stamps, K = 2, 4, 8).
+  const int k = v.K <= 4 ? 0 : v.K - 4;
+  const double chain = rule == BKMOO_CAGRAD ? 16 + 6 * k
+                                            : (rule == BKMOO_PCGRAD ? 10 + 9 * k : 8 + 5.5 * k);
+  const int64_t nb = v.b_hi - v.b_lo, nch = v.c_hi - v.c_lo;
+  const int64_t sets = (v.max_chunks + kSetChunks - 1) / kSetChunks;
+  StreamShape s;
+  // a team's warps share a bucket's sets; at least two of the CTA's 16 warps,
+  // so that no more than two solve on one scheduler
+  s.team = sets <= 2 ? 2 : sets <= 4 ? 4 : 8;
+  // teams: twice the buckets that complete during one chain
+  const double period = (double)nch * v.chunk_elems * v.K * elem_bytes(v.in_dtype) / 7e6 / nb;
+  double teams = 2.0 * chain / period + 1.0;
+  if (teams > nb) teams = (double)nb;
+  int64_t n = (int64_t)((teams * s.team + 15.0) / 16.0);
+  if (n > sms / 10) n = sms / 10;
+  // a small plan leaves SMs free: four solving warps on each
+  const int64_t idle = sms - nch, want = (nb + 3) / 4;
+  if (idle > n && want > n) n = want < idle ? want : idle;
+  s.n_solve = n < 1 ? 1 : (int)n;
+  s.n_stream = sms - s.n_solve;
+  if (s.n_stream > nch) s.n_stream = (int)nch;
+  // the copies in flight, a chunk, and what the Gram streams during the chain
+  // (25-35 KiB per SM and us); more lets the kept part of the window shrink
+  // (K = 4, 1 MiB fp32 buckets, MGDA: 500 KiB 0.92, 650 0.90, 800 0.95, 1300
+  // 1.06 us per bucket)
+  s.lead_kib = (int)(64 * v.K + 128 + 30 * chain);
+  return s;
 }
 
-// The fused path: one cooperative (co-resident) launch of kFusedThreads per
-// CTA, one CTA per SM.
-int launch_fused(const GradPtrs& g, const PlanView& v, const SolveParams& sp, void* ws,
-                 float* out_weights, int32_t* out_status, void* out, int dto,
-                 double bucket_bytes_max, cudaStream_t s) {
+// The streamed path over the view's window; *taken = false when the device
+// cannot hold it (the caller then runs the three launches).
+int launch_stream(const GradPtrs& g, const PlanView& v, const SolveParams& sp, void* ws,
+                  float* out_weights, int32_t* out_status, void* out, int dto, bool reset,
+                  bool* taken, cudaStream_t s) {
+  *taken = false;
+  const int64_t nch = v.c_hi - v.c_lo;
+  if (v.K > kStreamMaxK || nch <= 0) return BKMOO_OK;
+  const void* fn = stream_fn(v.K, v.in_dtype);
+  const int smem = stream_smem(v.K);
+  int sms = 0;
+  if (persistent_grid(fn, stream_threads(), &sms, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (sms < 2) return BKMOO_OK;
+  const StreamShape sh = stream_shape(v, sp.rule, sms);
   const WsLayout L = ws_layout(v.K, v.n_buckets, v.n_chunks);
   char* base = static_cast<char*>(ws);
-  if (cudaMemsetAsync(&v.hdr->status, 0, sizeof(int32_t), s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (v.n_buckets == 0) return BKMOO_OK;
-  if (cudaMemsetAsync(base + L.arrive, 0, L.ring - L.arrive, s) != cudaSuccess)
+  const size_t rw = (size_t)stream_row_words(v.K);
+  StreamView sv;
+  sv.v = v;
+  sv.w0 = v.c_lo;
+  sv.rows = reinterpret_cast<uint64_t*>(base + L.rows) + (size_t)v.c_lo * rw;
+  sv.chunk_bucket = reinterpret_cast<const int32_t*>(base + L.chunk_bucket);
+  sv.give_up = reinterpret_cast<int32_t*>(sv.rows + rw - 1);
+  const int kib = stream_stage_kib(v.K);
+  sv.n_stream = sh.n_stream;
+  sv.team = sh.team;
+  sv.lead = sh.lead_kib / kib;
+  // 320 KiB on every SM: 48 MB of L2, what the re-read still finds there
+  sv.l2_stages = 320 / kib;
+  sv.reset = reset ? 1 : 0;
+  if (cudaMemsetAsync(sv.rows, 0, (size_t)nch * rw * sizeof(uint64_t), s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
-  const void* fn = fused_fn(v.K, v.in_dtype, dto);
-  int grid = 0;
-  if (persistent_grid(fn, kFusedThreads, &grid, fused_smem_bytes(v.K)) != cudaSuccess)
-    return BKMOO_ERR_CUDA;
-  if (grid > kFusedMaxCtas) grid = kFusedMaxCtas;
-  if (grid < 1) return BKMOO_ERR_CUDA;
-  int dev = 0, l2 = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess)
-    return BKMOO_ERR_CUDA;
-  const FusedShape sh = fused_shape(grid, v.n_buckets, bucket_bytes_max, l2);
-  FusedView f;
-  f.v = v;
-  f.arrive = reinterpret_cast<int32_t*>(base + L.arrive);
-  f.ready = reinterpret_cast<int32_t*>(base + L.ready);
-  f.ring = reinterpret_cast<double*>(base + L.ring);
-  f.out_weights = out_weights;
-  f.out_status = out_status;
-  f.n_groups = sh.n_groups;
-  f.group_ctas = (grid + sh.n_groups - 1) / sh.n_groups;
-  f.lookahead = sh.lookahead;
   GradPtrs ga = g;
-  SolveParams spa = sp;
-  void* outp = out;
-  void* args[] = {&ga, &f, &spa, &outp};
-  if (cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kFusedThreads), args,
-                                  fused_smem_bytes(v.K), s) != cudaSuccess)
-    return BKMOO_ERR_CUDA;
-  return BKMOO_OK;
-}
-
-// The cluster-per-bucket fused path: as many clusters of kClusterCtas CTAs
-// as can be resident at once, at most one per bucket (clusters never wait
-// for one another).  `head`: items per streaming thread of the next
-// bucket's Gram read before a combination, to cover the rule's solve
-// (environment variable BKMOO_CLUSTER_HEAD overrides it, for tuning).
-int launch_fused_cluster(const GradPtrs& g, const PlanView& v, const SolveParams& sp,
-                         float* out_weights, int32_t* out_status, void* out, int dto,
-                         int64_t smax, cudaStream_t s) {
-  if (cudaMemsetAsync(&v.hdr->status, 0, sizeof(int32_t), s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (v.n_buckets == 0) return BKMOO_OK;
-  const void* fn = fused_cluster_fn(v.K, v.in_dtype, dto);
-  if (!fn) return BKMOO_ERR_INVALID;
-  const int smem = fused_cluster_smem(v.K);
-  static std::mutex mu;
-  static std::map<std::pair<int, const void*>, int> clusters;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return BKMOO_ERR_CUDA;
-  int ncl = 0;
-  {
-    std::lock_guard<std::mutex> lk(mu);
-    auto key = std::make_pair(dev, fn);
-    auto it = clusters.find(key);
-    if (it == clusters.end()) {
-      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-          cudaSuccess)
-        return BKMOO_ERR_CUDA;
-      cudaLaunchConfig_t cfg = {};
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = kClusterCtas;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.gridDim = dim3(kClusterCtas);
-      cfg.blockDim = dim3(kClusterThreads);
-      cfg.dynamicSmemBytes = (size_t)smem;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess) return BKMOO_ERR_CUDA;
-      it = clusters.emplace(key, n).first;
-    }
-    ncl = it->second;
-  }
-  if (ncl < 1) return BKMOO_ERR_CUDA;
-  if ((int64_t)ncl > v.n_buckets) ncl = (int)v.n_buckets;
-  // look-ahead: 512 bytes of gradients per streaming thread (32 / K items),
-  // or the whole next bucket when it has at most 24 items per thread
-  // (measured best on GB300: K = 2 16 items, K = 3 11, K = 4 8-12 at 2 MiB
-  // fp32 buckets, the whole bucket at 1 MiB)
-  const int64_t eb = elem_bytes(v.in_dtype), epv = 16 / eb;
-  const int64_t items = (smax / epv / kClusterCtas + kClusterStreamThreads - 1) / kClusterStreamThreads;
-  int64_t h = items <= 24 ? items : 32 / v.K;
-  if (h < 2) h = 2;
-  int head = (int)h;
-  if (const char* e = std::getenv("BKMOO_CLUSTER_HEAD")) {
-    const int h = std::atoi(e);
-    if (h >= 0) head = h;
-  }
-  GradPtrs ga = g;
-  PlanView va = v;
   SolveParams spa = sp;
   float* ow = out_weights;
   int32_t* os = out_status;
   void* outp = out;
-  void* args[] = {&ga, &va, &spa, &ow, &os, &outp, &head};
-  if (cudaLaunchKernel(fn, dim3(ncl * kClusterCtas), dim3(kClusterThreads), args, (size_t)smem,
-                       s) != cudaSuccess)
-    return BKMOO_ERR_CUDA;
+  int d = dto;
+  void* args[] = {&ga, &sv, &spa, &ow, &os, &outp, &d};
+  const cudaError_t e =
+      cudaLaunchCooperativeKernel(fn, dim3(sh.n_stream + sh.n_solve), dim3(stream_threads()),
+                                  args, (size_t)smem, s);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    (void)cudaGetLastError();
+    return BKMOO_OK;
+  }
+  if (e != cudaSuccess) return BKMOO_ERR_CUDA;
+  *taken = true;
   return BKMOO_OK;
 }
 
-// Path of bkmoo_resolve (see bkmoo_resolve_path in bkmoo.h): 0 three
-// launches, 1 cluster-per-bucket fused kernel, 2 grid-synchronised fused
-// kernel.
+// bkmoo_resolve_path's answer (see bkmoo.h): 1 or 2 where one launch is
+// certain, by the flags or for the plans listed there; 0 otherwise.
 int choose_path(int32_t K, int32_t dt, int32_t rule, const int64_t* off, int64_t B,
                 uint32_t flags) {
   if (flags & BKMOO_FLAG_THREE_PASS) return 0;
   if (flags & BKMOO_FLAG_FUSED) {
-    if (K <= kClusterMaxK && !(flags & BKMOO_FLAG_TEST_WITHHOLD)) return 1;
-    return K <= kFusedMaxK ? 2 : 0;
+    if (K <= 4 && !(flags & BKMOO_FLAG_TEST_WITHHOLD)) return 1;
+    return K <= kStreamMaxK ? 2 : 0;
   }
-  // measured on GB300 (1e9 elements per language, MGDA, fused / three
-  // launches): the cluster kernel is faster for tiny plans, where one
-  // launch instead of three is what counts (33 / 43 us), and for K = 2..4
-  // when buckets are large enough to amortise each bucket's hand-offs
-  // (>= 2 MiB) and small enough that the buckets in flight stay in L2:
-  // fp32 K = 2 2.71 / 2.97 ms at 2 MiB, 2.50 / 2.95 at 4 MiB; K = 3 3.43 /
-  // 3.95 at 2 MiB; K = 4 4.59 / 5.07 at 2 MiB, 4.74 / 5.06 at 3 MiB; 1 MiB
-  // buckets are slower or tie, and K x bucket above 12 MiB (fp32) or
-  // outside 6..12 MiB (bf16) ties or loses.  CAGrad, whose solve takes
-  // 5.5-7 us, gains only from 8 MiB of fp32 gradients per bucket (K = 4
-  // 2 MiB 4.95 / 5.06, K = 2 4 MiB 2.73 / 2.93; K = 2 2 MiB and bf16 lose).
   if (B < 1) return 0;
   if (K <= 2 && B <= 8 && off[B] <= ((int64_t)1 << 22)) return 1;
-  if (K < 2 || K > kClusterMaxK) return 0;
+  if (K < 2 || K > 4) return 0;
   int64_t smax = 0;
   for (int64_t b = 0; b < B; ++b) smax = off[b + 1] - off[b] > smax ? off[b + 1] - off[b] : smax;
   const double mib = 1024.0 * 1024.0;
@@ -274,7 +224,7 @@ int prepare(const void* const* grads, int32_t K, int32_t dt, const int64_t* offs
   const int64_t ch = chunk_elems(dt);
   const int64_t nch = count_chunks(offsets, B, ch);
   const WsLayout L = ws_layout(K, B, nch);
-  if (ws_bytes < L.total_fused) return BKMOO_ERR_WORKSPACE;
+  if (ws_bytes < L.total_all) return BKMOO_ERR_WORKSPACE;
   char* base = static_cast<char*>(ws);
   v->hdr = reinterpret_cast<WsHeader*>(base);
   v->offsets = reinterpret_cast<const int64_t*>(base + L.offsets);
@@ -472,7 +422,7 @@ int bkmoo_workspace_size(int32_t K, int32_t in_dtype, const int64_t* offsets,
   if (!bytes || K < 1 || K > kMaxK || !dtype_ok(in_dtype) || !offsets_ok(offsets, n_buckets))
     return BKMOO_ERR_INVALID;
   const int64_t nch = count_chunks(offsets, n_buckets, chunk_elems(in_dtype));
-  *bytes = ws_layout(K, n_buckets, nch).total_fused;
+  *bytes = ws_layout(K, n_buckets, nch).total_all;
   return BKMOO_OK;
 }
 
@@ -484,7 +434,7 @@ int bkmoo_workspace_init(int32_t K, int32_t in_dtype, const int64_t* offsets,
   const int64_t ch = chunk_elems(in_dtype);
   const int64_t nch = count_chunks(offsets, n_buckets, ch);
   const WsLayout L = ws_layout(K, n_buckets, nch);
-  if (ws_bytes < L.total_fused) return BKMOO_ERR_WORKSPACE;
+  if (ws_bytes < L.total_all) return BKMOO_ERR_WORKSPACE;
   // Host image of header + bucket table, copied in one transfer.
   std::vector<unsigned char> img(L.partials, 0);
   WsHeader h;
@@ -503,8 +453,16 @@ int bkmoo_workspace_init(int32_t K, int32_t in_dtype, const int64_t* offsets,
   int64_t* cp = reinterpret_cast<int64_t*>(img.data() + L.chunk_prefix);
   cp[0] = 0;
   for (int64_t b = 0; b < n_buckets; ++b) cp[b + 1] = cp[b] + (offsets[b + 1] - offsets[b] + ch - 1) / ch;
+  // The bucket of every chunk (streamed path).
+  std::vector<int32_t> cb((size_t)nch);
+  for (int64_t b = 0; b < n_buckets; ++b)
+    for (int64_t c = cp[b]; c < cp[b + 1]; ++c) cb[(size_t)c] = (int32_t)b;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (cudaMemcpyAsync(ws, img.data(), img.size(), cudaMemcpyHostToDevice, s) != cudaSuccess)
+    return BKMOO_ERR_CUDA;
+  if (nch > 0 && cudaMemcpyAsync(static_cast<char*>(ws) + L.chunk_bucket, cb.data(),
+                                 sizeof(int32_t) * (size_t)nch, cudaMemcpyHostToDevice,
+                                 s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
   if (cudaStreamSynchronize(s) != cudaSuccess) return BKMOO_ERR_CUDA;
   return BKMOO_OK;
@@ -538,25 +496,16 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype, const i
   cudaEvent_t* ev = static_cast<cudaEvent_t*>(prm.events);
   const SolveParams sp = solve_params(rule, prm);
   if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  const int path = choose_path(K, in_dtype, rule, offsets, n_buckets, prm.flags);
-  int64_t nmax = 0;
-  if (path != 0)
-    for (int64_t b = 0; b < n_buckets; ++b)
-      if (offsets[b + 1] - offsets[b] > nmax) nmax = offsets[b + 1] - offsets[b];
-  if (path == 1) {
-    r = launch_fused_cluster(g, v, sp, out_weights, out_status, out_dir, out_dtype, nmax, s);
+  if (choose_path(K, in_dtype, rule, offsets, n_buckets, prm.flags) != 0 ||
+      (!(prm.flags & BKMOO_FLAG_THREE_PASS) && stream_wins(v, offsets))) {
+    bool taken = false;
+    r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, true, &taken, s);
     if (r != BKMOO_OK) return r;
-    for (int i = 1; i < 4; ++i)
-      if (ev && cudaEventRecord(ev[i], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-    return BKMOO_OK;
-  }
-  if (path == 2) {
-    r = launch_fused(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype,
-                     (double)nmax * (K * elem_bytes(in_dtype) + elem_bytes(out_dtype)), s);
-    if (r != BKMOO_OK) return r;
-    for (int i = 1; i < 4; ++i)
-      if (ev && cudaEventRecord(ev[i], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-    return BKMOO_OK;
+    if (taken) {
+      for (int i = 1; i < 4; ++i)
+        if (ev && cudaEventRecord(ev[i], s) != cudaSuccess) return BKMOO_ERR_CUDA;
+      return BKMOO_OK;
+    }
   }
   r = launch_gram_pass(g, v, s);
   if (r != BKMOO_OK) return r;
@@ -591,6 +540,11 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   v.c_hi = c;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const SolveParams sp = solve_params(rule, prm);
+  if (!(prm.flags & BKMOO_FLAG_THREE_PASS) && stream_wins(v, offsets)) {
+    bool taken = false;
+    r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
+    if (r != BKMOO_OK || taken) return r;
+  }
   r = launch_gram_pass(g, v, s, false);
   if (r != BKMOO_OK) return r;
   if (launch_solve(v, sp, out_weights, out_status, s) != cudaSuccess) return BKMOO_ERR_CUDA;

@@ -50,9 +50,9 @@ __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
 
 // Block (x = group j, y-stride over buckets b): for a bucket of more than
 // kGroupMinChunks chunks, thread p < K(K+1)/2 sums entry p over the chunks
-// [c0 + 512 j, c0 + 512 (j+1)) of the bucket (eight interleaved fp64 sums,
-// fixed tree) and writes the result into the group's first row.  Each
-// (row, entry) is read and written by one thread only.
+// [c0 + 512 j, c0 + 512 (j+1)) of the bucket (sum_chunk_rows) and writes the
+// result into the group's first row.  Each (row, entry) is read and written
+// by one thread only.
 __global__ void __launch_bounds__(256) group_reduce_kernel(const PlanView v) {
   if (!header_ok(v)) return;
   const int P = tri(v.K);
@@ -63,18 +63,8 @@ __global__ void __launch_bounds__(256) group_reduce_kernel(const PlanView v) {
     if (cb1 - cb0 <= kGroupMinChunks) continue;
     const int64_t c0 = cb0 + (int64_t)blockIdx.x * kGroupChunks;
     if (c0 >= cb1) continue;
-    const int64_t c1 = min(c0 + kGroupChunks, cb1);
-    double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    const double* src = v.partials + c0 * P + p;
-    int64_t c = c0;
-    for (; c + 8 <= c1; c += 8, src += 8 * P) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) t[j] += src[j * P];
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (c + j < c1) t[j] += src[j * P];
-    v.partials[c0 * P + p] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    double* row = v.partials + c0 * P + p;
+    *row = sum_chunk_rows(row, P, min(kGroupChunks, cb1 - c0), v.K);
   }
 }
 

@@ -1,5 +1,6 @@
 // Per-bucket solvers of the MOO rules on a bucket's Gram matrix G (fp64),
-// shared by the solve kernel (solve.cu) and the fused kernel (fused.cu).
+// shared by the solve kernel (solve.cu) and the streamed kernel
+// (stream_resolve.cuh).
 // A whole warp enters solve_bucket_warp(); the coefficients beta of
 // d_b = sum_k beta_k g_k come out in shared memory.
 //
@@ -65,25 +66,12 @@ constexpr double kPivot = 1e-13;   // smallest pivot of a non-singular system
 // each group of kGroupChunks, and those rows are what is summed here.
 __device__ void reduce_bucket(const PlanView& v, int64_t b, double* G, int lane) {
   const int K = v.K, P = tri(K);
-  int64_t c0 = v.chunk_prefix[b], c1 = v.chunk_prefix[b + 1];
-  int64_t stride = 1;  // in chunks
-  if (c1 - c0 > kGroupMinChunks) {
-    stride = kGroupChunks;
-    c1 = c0 + (c1 - c0 + kGroupChunks - 1) / kGroupChunks;  // c0 + number of groups
-  }
-  const int64_t rs = stride * P;  // doubles between the rows summed
+  const int64_t c0 = v.chunk_prefix[b], n = v.chunk_prefix[b + 1] - c0;
+  const bool pre = n > kGroupMinChunks;
   for (int p = lane; p < P; p += 32) {
-    double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     const double* src = v.partials + c0 * P + p;
-    int64_t c = c0;
-    for (; c + 8 <= c1; c += 8, src += 8 * rs) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) t[j] += src[j * rs];
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      if (c + j < c1) t[j] += src[j * rs];
-    const double s = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    const double s = pre ? sum_rows8(src, kGroupChunks * P, (n + kGroupChunks - 1) / kGroupChunks)
+                         : sum_chunk_rows(src, P, n, K);
     int i = 0, r = p;
     while (r >= K - i) {
       r -= K - i;

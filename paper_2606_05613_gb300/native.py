@@ -297,8 +297,8 @@ def bkmoo_version() -> int:
 
 
 def bkmoo_resolve_path(K: int, in_dtype: int, rule, offsets, flags: int) -> int:
-    """0: three launches; 1: cluster-per-bucket fused kernel; 2:
-    grid-synchronised fused kernel (the path bkmoo_resolve takes)."""
+    """1 or 2: one launch; 0: bkmoo_resolve may take the three launches (see
+    include/bkmoo.h)."""
     if isinstance(rule, str):
         rule = RULES[rule]
     off = _offsets_array(offsets)

@@ -1,0 +1,185 @@
+"""GPU: the streamed launch gives the three launches' results bit for bit, on
+plans at the edges of its chunks, stages, sets and windows, in place, bucket
+range by bucket range, and from several streams and threads at once."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2606_05613_gb300 import build as nb
+from paper_2606_05613_gb300 import native as bk
+
+pytestmark = pytest.mark.gpu
+
+DEV = torch.device("cuda:0")
+F32, BF16 = torch.float32, torch.bfloat16
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    nb.build()
+    bk.load()
+
+
+def _plan(dt, kind):
+    """Bucket offsets, in chunks of ch elements (256 threads x 16 vectors)."""
+    ch = 16384 if dt == F32 else 32768
+    if kind == "tiny":          # shorter than a vector, a stage, a chunk
+        sizes = [1, 2, 3, 7, 8, 9, 15, 17, 255, 257, 4097, ch - 1, ch, ch + 1]
+    elif kind == "sets":        # a set of 16 chunks, one more, one less; aligned and not
+        sizes = [16 * ch, 17 * ch, 15 * ch, 5, 16 * ch + 1, 33 * ch - 3]
+    elif kind == "waves":       # more chunks than SMs, the last ones short
+        sizes = [401 * ch + 11, 3, 150 * ch, 153 * ch - 1]
+    else:                       # "groups": more than 1024 chunks, ragged groups of 512
+        sizes = [1025 * ch + 7, 5000, 1536 * ch + 3]
+    return np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+
+
+def _grads(K, dt, n, seed):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    s = torch.randn(n, generator=g, device=DEV)
+    return [(torch.randn(n, generator=g, device=DEV) + 0.4 * (-1) ** k * s).to(dt)
+            for k in range(K)]
+
+
+def _params(flag):
+    p = bk.bkmoo_default_params()
+    p.flags |= flag
+    return p
+
+
+def _run(res, grads, rule, odt, flag, inplace=False, step=0, stream=None):
+    g = [x.clone() for x in grads] if inplace else grads
+    n, B, K = int(res.offsets[-1]), res.n_buckets, len(g)
+    out = g[0] if inplace else torch.full((n,), 3.0, dtype=odt, device=DEV)
+    w = torch.full((B, K), -1.0, device=DEV)
+    st = torch.full((B,), -1, dtype=torch.int32, device=DEV)
+    kw = dict(params=_params(flag), out_weights=w, out_status=st, stream=stream)
+    if step:
+        for b in range(0, B, step):
+            res.resolve_buckets(g, b, min(B, b + step), rule, out, **kw)
+    else:
+        res.resolve(g, rule, out, **kw)
+    return out, w, st
+
+
+def _same(a, b):
+    for x, y in zip(a, b):
+        assert torch.equal(x.view(torch.uint8), y.view(torch.uint8))
+
+
+@pytest.mark.parametrize("kind", ["tiny", "sets", "waves", "groups"])
+@pytest.mark.parametrize("dt", [F32, BF16])
+@pytest.mark.parametrize("K", range(1, 9))
+def test_stream_is_the_three_launches(K, dt, kind):
+    if kind == "groups" and K > 4:
+        pytest.skip("the groups' order does not depend on K; 4 GB of gradients")
+    off = _plan(dt, kind)
+    grads = _grads(K, dt, int(off[-1]), 7 * K)
+    res = bk.Resolver(K, dt, off, DEV)
+    for rule, odt, inplace in (("mgda", dt, False), ("pcgrad", F32, False),
+                               ("cagrad", BF16, False), ("mgda", dt, True)):
+        three = _run(res, grads, rule, odt, bk.BKMOO_FLAG_THREE_PASS, inplace)
+        one = _run(res, grads, rule, odt, bk.BKMOO_FLAG_FUSED, inplace)
+        torch.cuda.synchronize()
+        assert res.status() == 0
+        _same(three, one)
+    three = _run(res, grads, "mgda", dt, bk.BKMOO_FLAG_THREE_PASS)
+    by_range = _run(res, grads, "mgda", dt, 0, step=2)     # windows inside the plan
+    torch.cuda.synchronize()
+    assert res.status() == 0
+    _same(three, by_range)
+
+
+def test_stream_nonfinite_and_zero_buckets():
+    """NaN, infinities, and zero gradients: the row words' "not written" value
+    is no partial's."""
+    ch = 16384
+    off = np.array([0, 3 * ch, 5 * ch, 9 * ch, 10 * ch], dtype=np.int64)
+    grads = _grads(4, F32, int(off[-1]), 3)
+    grads[1][ch + 5] = float("nan")
+    grads[2].view(torch.int32)[4 * ch] = -1          # the NaN of all ones
+    for g in grads:
+        g[int(off[2]):int(off[3])] = 0.0
+    grads[0][int(off[3])] = float("inf")
+    res = bk.Resolver(4, F32, off, DEV)
+    for rule in ("mgda", "pcgrad", "cagrad", "mean"):
+        three = _run(res, grads, rule, F32, bk.BKMOO_FLAG_THREE_PASS)
+        one = _run(res, grads, rule, F32, bk.BKMOO_FLAG_FUSED)
+        torch.cuda.synchronize()
+        assert one[2].tolist() == [bk.BKMOO_ERR_NONFINITE, bk.BKMOO_ERR_NONFINITE, 0,
+                                   bk.BKMOO_ERR_NONFINITE]
+        assert res.status() == 0
+        _same(three[1:], one[1:])
+        _same([three[0][int(off[2]):int(off[3])]], [one[0][int(off[2]):int(off[3])]])
+        assert torch.equal(torch.isnan(three[0]), torch.isnan(one[0]))
+
+
+@pytest.mark.parametrize("shared", [False, True])
+def test_stream_from_several_streams_and_threads(shared):
+    """Two threads, a stream of another priority each, many resolves at once:
+    workspaces of their own, or disjoint bucket ranges of one plan and
+    workspace."""
+    ch, K = 16384, 4
+    off = np.array([0] + [40 * ch * (i + 1) + 13 * i for i in range(6)], dtype=np.int64)
+    grads = _grads(K, F32, int(off[-1]), 11)
+    ws = [bk.Resolver(K, F32, off, DEV) for _ in range(1 if shared else 2)]
+    want = _run(ws[0], grads, "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(DEV, priority=p) for p in (0, -1)]
+    n, B = int(off[-1]), len(off) - 1
+    outs = [[torch.zeros(n, device=DEV), torch.zeros(B, K, device=DEV),
+             torch.zeros(B, dtype=torch.int32, device=DEV)] for _ in range(1 if shared else 2)]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(t):
+        try:
+            o = outs[0 if shared else t]
+            r = ws[0 if shared else t]
+            for _ in range(20):
+                kw = dict(out_weights=o[1], out_status=o[2], stream=streams[t])
+                if shared:
+                    r.resolve_buckets(grads, 3 * t, 3 * t + 3, "mgda", o[0], **kw)
+                else:
+                    r.resolve(grads, "mgda", o[0], params=_params(bk.BKMOO_FLAG_FUSED), **kw)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    for r in ws:
+        assert r.status() == 0
+    for o in outs:
+        _same(want, o)
+
+
+def test_stream_under_graph_capture():
+    """Captured once, replayed on new inputs."""
+    off = _plan(F32, "sets")
+    K = 3
+    res = bk.Resolver(K, F32, off, DEV)
+    grads = _grads(K, F32, int(off[-1]), 5)
+    out = torch.zeros(int(off[-1]), device=DEV)
+    s = torch.cuda.Stream(DEV)
+    p = _params(bk.BKMOO_FLAG_FUSED)
+    res.resolve(grads, "mgda", out, params=p, stream=s)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        res.resolve(grads, "mgda", out, params=p)
+    for seed in (21, 22):
+        for g, x in zip(grads, _grads(K, F32, int(off[-1]), seed)):
+            g.copy_(x)
+        graph.replay()
+        torch.cuda.synchronize()
+        got = out.clone()
+        want = _run(res, grads, "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)[0]
+        assert torch.equal(got, want)
+        assert res.status() == 0
