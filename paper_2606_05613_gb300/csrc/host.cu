@@ -540,7 +540,11 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   v.c_hi = c;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const SolveParams sp = solve_params(rule, prm);
-  if (!(prm.flags & BKMOO_FLAG_THREE_PASS) && stream_wins(v, offsets)) {
+  // One or two buckets: the three launches, which share the SMs with whatever
+  // the caller overlaps them with; the streamed launch needs all of them at
+  // once (a training step that resolves each bucket beside the backward pass:
+  // 263.9 ms with three launches per bucket, 267.3 streamed).
+  if (!(prm.flags & BKMOO_FLAG_THREE_PASS) && b_hi - b_lo > 2 && stream_wins(v, offsets)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
     if (r != BKMOO_OK || taken) return r;

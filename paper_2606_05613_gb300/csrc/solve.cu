@@ -35,6 +35,52 @@ __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
   if (lane == 0 && out_status) out_status[b] = st;
 }
 
+// One block of eight warps per bucket, for plans with buckets of many chunks:
+// the rows of a bucket are then the longest part of the pass (one warp adds
+// them at one fp64 instruction per 64 cycles; a 400-chunk K = 4 bucket: 68 -> 60
+// us for the three launches of the bucket alone).
+__global__ void __launch_bounds__(32 * kWideWarps)
+    solve_wide_kernel(const PlanView v, const SolveParams p, float* out_weights,
+                      int32_t* out_status) {
+  __shared__ double t8[kWideWarps * tri(kMaxK)];
+  __shared__ double G[kMaxK * kMaxK];
+  __shared__ double beta[kMaxK];
+  __shared__ float Gf[kMaxK * kMaxK];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t b = v.b_lo + blockIdx.x;
+  const int K = v.K;
+  if (!header_ok(v)) {
+    if (threadIdx.x == 0 && out_status) out_status[b] = BKMOO_ERR_WORKSPACE;
+    return;
+  }
+  reduce_bucket_wide(v, b, t8, lane, w);
+  __syncthreads();
+  if (w != 0) return;
+  gram_from_sums(K, t8, G, lane);
+  const int st = solve_bucket_warp<0>(K, G, Gf, p, b, beta, lane);
+  for (int k = lane; k < K; k += 32) {
+    const float f = (float)beta[k];
+    v.beta[b * K + k] = f;
+    if (out_weights) out_weights[b * K + k] = f;
+  }
+  if (lane == 0 && out_status) out_status[b] = st;
+}
+
+__global__ void __launch_bounds__(32 * kWideWarps)
+    gram_finalize_wide_kernel(const PlanView v, double* out_gram) {
+  __shared__ double t8[kWideWarps * tri(kMaxK)];
+  __shared__ double G[kMaxK * kMaxK];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t b = blockIdx.x;
+  if (!header_ok(v)) return;
+  const int K = v.K;
+  reduce_bucket_wide(v, b, t8, lane, w);
+  __syncthreads();
+  if (w != 0) return;
+  gram_from_sums(K, t8, G, lane);
+  for (int i = lane; i < K * K; i += 32) out_gram[b * K * K + i] = G[i];
+}
+
 __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
     gram_finalize_kernel(const PlanView v, double* out_gram) {
   __shared__ double Gs[kSolveWarpsPerBlock][kMaxK * kMaxK];
@@ -97,9 +143,18 @@ cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Buckets of more chunks than this take a block each (below, a warp adds the
+// rows in the time that the block's hand-off takes).
+constexpr int64_t kWideMinChunks = 32;
+
 cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_weights,
                          int32_t* out_status, cudaStream_t s) {
   if (v.b_hi <= v.b_lo) return cudaSuccess;
+  if (v.max_chunks > kWideMinChunks) {
+    solve_wide_kernel<<<(unsigned)(v.b_hi - v.b_lo), 32 * kWideWarps, 0, s>>>(v, p, out_weights,
+                                                                             out_status);
+    return cudaGetLastError();
+  }
   const int64_t grid = (v.b_hi - v.b_lo + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
   solve_kernel<<<(unsigned)grid, 32 * kSolveWarpsPerBlock, 0, s>>>(v, p, out_weights, out_status);
   return cudaGetLastError();
@@ -107,6 +162,10 @@ cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_wei
 
 cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s) {
   if (v.n_buckets == 0) return cudaSuccess;
+  if (v.max_chunks > kWideMinChunks) {
+    gram_finalize_wide_kernel<<<(unsigned)v.n_buckets, 32 * kWideWarps, 0, s>>>(v, out_gram);
+    return cudaGetLastError();
+  }
   const int64_t grid = (v.n_buckets + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
   gram_finalize_kernel<<<(unsigned)grid, 32 * kSolveWarpsPerBlock, 0, s>>>(v, out_gram);
   return cudaGetLastError();

@@ -84,6 +84,67 @@ __device__ void reduce_bucket(const PlanView& v, int64_t b, double* G, int lane)
   __syncwarp();
 }
 
+// The same by a block of eight warps, for buckets of many chunks: warp w forms
+// the interleaved sum w of every entry (t8: [8][P] in shared memory), which
+// the caller adds by tree8_entry once the block has synchronised.
+constexpr int kWideWarps = 8;
+__device__ void reduce_bucket_wide(const PlanView& v, int64_t b, double* t8, int lane, int w) {
+  const int K = v.K, P = tri(K);
+  const int64_t c0 = v.chunk_prefix[b], n0 = v.chunk_prefix[b + 1] - c0;
+  const bool pre = n0 > kGroupMinChunks;
+  const int64_t n = pre ? (n0 + kGroupChunks - 1) / kGroupChunks : n0;
+  const int64_t rs = pre ? kGroupChunks * P : P;
+  const double* src = v.partials + c0 * P;
+  if (K <= kStreamMaxK && !pre) {
+    for (int p = lane; p < P; p += 32) {
+      double t = 0.0;
+      for (int64_t at = (int64_t)w * kSetChunks; at < n; at += kWideWarps * kSetChunks)
+        t += set_sum(src + at * rs + p, rs, n - at);
+      t8[w * P + p] = t;
+    }
+    return;
+  }
+  // rows w, w + 8, ...: four rows of up to five entries a lane in flight
+  constexpr int E = (tri(kMaxK) + 31) / 32, U = 4;
+  double t[E] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  static_assert(E == 5, "entries per lane");
+  for (int64_t c = w; c < n; c += kWideWarps * U) {
+    double x[U][E];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        x[u][e] = (c + u * kWideWarps < n && lane + 32 * e < P)
+                      ? src[(c + u * kWideWarps) * rs + lane + 32 * e]
+                      : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (c + u * kWideWarps < n && 32 * e < P) t[e] += x[u][e];
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane + 32 * e < P) t8[w * P + lane + 32 * e] = t[e];
+}
+// One warp: G from the eight interleaved sums.
+__device__ void gram_from_sums(int K, const double* t8, double* G, int lane) {
+  const int P = tri(K);
+  for (int p = lane; p < P; p += 32) {
+    const double* t = t8 + p;
+    const double s = ((t[0] + t[P]) + (t[2 * P] + t[3 * P])) +
+                     ((t[4 * P] + t[5 * P]) + (t[6 * P] + t[7 * P]));
+    int i = 0, r = p;
+    while (r >= K - i) {
+      r -= K - i;
+      ++i;
+    }
+    G[i * K + i + r] = s;
+    G[(i + r) * K + i] = s;
+  }
+  __syncwarp();
+}
+
 // ---------------------------------------------------------------------------
 // small dense helpers (lane 0 only)
 // ---------------------------------------------------------------------------

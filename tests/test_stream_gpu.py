@@ -86,7 +86,7 @@ def test_stream_is_the_three_launches(K, dt, kind):
         assert res.status() == 0
         _same(three, one)
     three = _run(res, grads, "mgda", dt, bk.BKMOO_FLAG_THREE_PASS)
-    by_range = _run(res, grads, "mgda", dt, 0, step=2)     # windows inside the plan
+    by_range = _run(res, grads, "mgda", dt, 0, step=3)     # windows inside the plan
     torch.cuda.synchronize()
     assert res.status() == 0
     _same(three, by_range)
