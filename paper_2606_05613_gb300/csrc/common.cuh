@@ -181,9 +181,37 @@ struct SolveParams {
   uint32_t flags;
 };
 
+// Launch that may begin before the kernel ahead of it in the stream has ended
+// (programmatic dependent launch): its CTAs are in place when that kernel's
+// last one leaves, instead of 2-4 us later.  Every kernel launched so waits at
+// its top (grid_wait) for that kernel's end, so an end implies the ends of all
+// before it.
+inline cudaError_t launch_behind(const void* fn, dim3 grid, dim3 block, void** args, size_t smem,
+                                 cudaStream_t s, bool behind) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = behind ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 // ---------------------------------------------------------------------------
 // Device helpers
 // ---------------------------------------------------------------------------
+
+// Until the kernels ahead in the stream have ended and their writes are
+// visible (nothing to wait for after a plain launch).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// From here on the next kernel's CTAs may be put beside this kernel's.
+__device__ __forceinline__ void grid_release() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ bool header_ok(const PlanView& v) {
   const WsHeader* h = v.hdr;
@@ -318,16 +346,13 @@ int gram_prefetch_min_k();
 
 // Combine kernels with a per-thread shared-memory prefetch (same signature,
 // combine_prefetch_smem(K) bytes of dynamic shared memory), every K;
-// combine_prefetch.cu, combine_prefetch_k9_16.cu.  Measured faster than
-// combine_kernel on GB300 (K = 2..8: 2-6.5 %).
-#ifndef BKMOO_COMBINE_PREFETCH
-#define BKMOO_COMBINE_PREFETCH 1
-#endif
+// combine_prefetch.cu, combine_prefetch_k9_16.cu.
 const void* combine_prefetch_fn(int K, int dti, int dto);
 const void* combine_prefetch_fn_k9_16(int K, int dti, int dto);
 int combine_prefetch_smem(int K);
 
-// Combine kernels, signature (GradPtrs, PlanView, void* out); combine_*.cu.
+// Combine kernels that take the last chunk first, for short windows,
+// signature (GradPtrs, PlanView, void* out); combine_*.cu.
 const void* combine_fn_f32(int K, int dtype_out);
 const void* combine_fn_bf16(int K, int dtype_out);
 
@@ -344,15 +369,16 @@ int stream_smem(int K);
 int stream_stage_kib(int K);
 
 // solve.cu
+// `behind`: launched behind the Gram pass (launch_behind).
 cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_weights,
-                         int32_t* out_status, cudaStream_t s);
-cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s);
+                         int32_t* out_status, cudaStream_t s, bool behind);
+cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s, bool behind);
 // The fp64 division / square-root helpers of the fast solvers, element-wise
 // (self-test of their accuracy against the correctly rounded operations).
 cudaError_t launch_selftest_fp64(int op, const double* a, const double* b, double* out, int64_t n,
                                  cudaStream_t s);
 // After a Gram pass over the view's window: the group pre-reduction of its
 // large buckets (a no-op when no bucket has more than kGroupMinChunks chunks).
-cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s);
+cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s, bool behind);
 
 }  // namespace bkmoo

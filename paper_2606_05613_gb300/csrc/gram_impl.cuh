@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(kThreads) gram_partials_kernel(const GradPtrs 
   constexpr int UNROLL = (K <= 8) ? 2 : 1;
   __shared__ float red[kWarps][P];
 
+  grid_release();
   if (!header_ok(v)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) record_error(v.hdr, BKMOO_ERR_WORKSPACE);
     return;

@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kThreads) gram_prefetch_kernel(const GradPtrs 
   uint4* slots = reinterpret_cast<uint4*>(pf_smem);
   auto slot = [&](int s, int k) -> uint4* { return slots + ((s * K + k) * kThreads + threadIdx.x); };
 
+  grid_release();
   if (!header_ok(v)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) record_error(v.hdr, BKMOO_ERR_WORKSPACE);
     return;

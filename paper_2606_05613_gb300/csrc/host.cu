@@ -133,7 +133,11 @@ StreamShape stream_shape(const PlanView& v, int rule, int sms) {
   // (25-35 KiB per SM and us); more lets the kept part of the window shrink
   // (K = 4, 1 MiB fp32 buckets, MGDA: 500 KiB 0.92, 650 0.90, 800 0.95, 1300
   // 1.06 us per bucket)
+  // and for buckets of more than a chunk per SM, which complete in waves of
+  // chunks, part of a chunk more (8 Qwen3-8B layers: 624 KiB 3353, 800 3291, 1200
+  // 3342 us)
   s.lead_kib = (int)(64 * v.K + 128 + 30 * chain);
+  if (nch > nb * sms) s.lead_kib += 44 * v.K;
   return s;
 }
 
@@ -164,8 +168,9 @@ int launch_stream(const GradPtrs& g, const PlanView& v, const SolveParams& sp, v
   sv.n_stream = sh.n_stream;
   sv.team = sh.team;
   sv.lead = sh.lead_kib / kib;
-  // 320 KiB on every SM: 48 MB of L2, what the re-read still finds there
-  sv.l2_stages = 320 / kib;
+  // 48-58 MB of L2 in all, what the re-read still finds there (K = 4, 1 MiB
+  // buckets: 256 KiB per SM 871, 320 841, 384 818 us; more finds no more)
+  sv.l2_stages = (v.K <= 4 ? 384 : 320) / kib;
   sv.reset = reset ? 1 : 0;
   if (cudaMemsetAsync(sv.rows, 0, (size_t)nch * rw * sizeof(uint64_t), s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
@@ -250,7 +255,10 @@ int prepare(const void* const* grads, int32_t K, int32_t dt, const int64_t* offs
 
 // Gram pass over the view's window; `reset` clears the workspace status word
 // first (once per call of the C ABI, not per window).
-int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool reset = true) {
+// `behind`: the kernels after this pass are launched behind it (not where an
+// event is recorded between them).
+int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool reset,
+                     bool behind) {
   if (reset && cudaMemsetAsync(&v.hdr->status, 0, sizeof(int32_t), s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
   const int64_t nch = v.c_hi - v.c_lo;
@@ -267,7 +275,7 @@ int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool 
   void* args[] = {&ga, &va};
   if (cudaLaunchKernel(fn, dim3(grid), dim3(kThreads), args, smem, s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
-  if (launch_group_reduce(v, s) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (launch_group_reduce(v, s, behind) != cudaSuccess) return BKMOO_ERR_CUDA;
   return BKMOO_OK;
 }
 
@@ -275,12 +283,16 @@ int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_
                    cudaStream_t s) {
   const int64_t nch = v.c_hi - v.c_lo;
   if (nch <= 0) return BKMOO_OK;
-  const bool pf = BKMOO_COMBINE_PREFETCH != 0;
-  const void* fn = pf ? combine_prefetch_fn(v.K, v.in_dtype, out_dtype)
-                      : combine_fn(v.K, v.in_dtype, out_dtype);
-  const int smem = pf ? combine_prefetch_smem(v.K) : 0;
-  int grid = 0;
-  if (persistent_grid(fn, kThreads, &grid, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
+  // A window of a few chunks per CTA: last chunk first, out of L2 (GPT-2 small
+  // bucket by bucket, 90 MB each, 1331 -> 1250 us).
+  const void* fn = combine_fn(v.K, v.in_dtype, out_dtype);
+  int smem = 0, grid = 0;
+  if (persistent_grid(fn, kThreads, &grid) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (nch > 4 * (int64_t)grid) {
+    fn = combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
+    smem = combine_prefetch_smem(v.K);
+    if (persistent_grid(fn, kThreads, &grid, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
+  }
   if (grid > nch) grid = (int)nch;
   PlanView va = v;
   GradPtrs ga = g;
@@ -476,9 +488,9 @@ int bkmoo_gram(const void* const* grads, int32_t K, int32_t in_dtype, const int6
   int r = prepare(grads, K, in_dtype, offsets, n_buckets, ws, ws_bytes, &v, &g);
   if (r != BKMOO_OK) return r;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  r = launch_gram_pass(g, v, s);
+  r = launch_gram_pass(g, v, s, true, true);
   if (r != BKMOO_OK) return r;
-  if (launch_gram_finalize(v, out_gram, s) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (launch_gram_finalize(v, out_gram, s, true) != cudaSuccess) return BKMOO_ERR_CUDA;
   return BKMOO_OK;
 }
 
@@ -507,10 +519,10 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype, const i
       return BKMOO_OK;
     }
   }
-  r = launch_gram_pass(g, v, s);
+  r = launch_gram_pass(g, v, s, true, !ev);
   if (r != BKMOO_OK) return r;
   if (ev && cudaEventRecord(ev[1], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (launch_solve(v, sp, out_weights, out_status, s) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (launch_solve(v, sp, out_weights, out_status, s, !ev) != cudaSuccess) return BKMOO_ERR_CUDA;
   if (ev && cudaEventRecord(ev[2], s) != cudaSuccess) return BKMOO_ERR_CUDA;
   r = launch_combine(g, v, out_dir, out_dtype, s);
   if (r != BKMOO_OK) return r;
@@ -549,9 +561,9 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
     if (r != BKMOO_OK || taken) return r;
   }
-  r = launch_gram_pass(g, v, s, false);
+  r = launch_gram_pass(g, v, s, false, true);
   if (r != BKMOO_OK) return r;
-  if (launch_solve(v, sp, out_weights, out_status, s) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (launch_solve(v, sp, out_weights, out_status, s, true) != cudaSuccess) return BKMOO_ERR_CUDA;
   return launch_combine(g, v, out_dir, out_dtype, s);
 }
 
@@ -666,8 +678,9 @@ int bkmoo_resolve_host(const void* const* host_grads, int32_t K, int32_t in_dtyp
     vw.c_hi = c_next;
     ok = ok && cudaStreamWaitEvent(s, in_ready[slot], 0) == cudaSuccess;
     if (win >= kHostSlots) ok = ok && cudaStreamWaitEvent(s, out_free[slot], 0) == cudaSuccess;
-    if (ok) r = launch_gram_pass(gw, vw, s, false);
-    ok = ok && r == BKMOO_OK && launch_solve(vw, sp, out_weights, out_status, s) == cudaSuccess;
+    if (ok) r = launch_gram_pass(gw, vw, s, false, true);
+    ok = ok && r == BKMOO_OK &&
+         launch_solve(vw, sp, out_weights, out_status, s, true) == cudaSuccess;
     if (ok) r = launch_combine(gw, vw, outw, out_dtype, s);
     ok = ok && r == BKMOO_OK && cudaEventRecord(in_free[slot], s) == cudaSuccess &&
          cudaEventRecord(out_ready[slot], s) == cudaSuccess;

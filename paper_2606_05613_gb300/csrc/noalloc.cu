@@ -187,7 +187,7 @@ extern "C" int bkmoo_gram_noalloc(const void* const* grads, int32_t K, int32_t i
   void* args[] = {&g, &v};
   if (cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kThreads), args, smem, s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
-  if (launch_group_reduce(v, s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (launch_gram_finalize(v, out_gram, s) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (launch_group_reduce(v, s, true) != cudaSuccess) return BKMOO_ERR_CUDA;
+  if (launch_gram_finalize(v, out_gram, s, true) != cudaSuccess) return BKMOO_ERR_CUDA;
   return BKMOO_OK;
 }

@@ -15,6 +15,7 @@ __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
   __shared__ double Gs[kSolveWarpsPerBlock][kMaxK * kMaxK];
   __shared__ double Bs[kSolveWarpsPerBlock][kMaxK];
   __shared__ float Fs[kSolveWarpsPerBlock][kMaxK * kMaxK];
+  grid_wait();
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int64_t b = v.b_lo + (int64_t)blockIdx.x * kSolveWarpsPerBlock + wi;
   if (b >= v.b_hi) return;
@@ -46,6 +47,7 @@ __global__ void __launch_bounds__(32 * kWideWarps)
   __shared__ double G[kMaxK * kMaxK];
   __shared__ double beta[kMaxK];
   __shared__ float Gf[kMaxK * kMaxK];
+  grid_wait();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t b = v.b_lo + blockIdx.x;
   const int K = v.K;
@@ -70,6 +72,7 @@ __global__ void __launch_bounds__(32 * kWideWarps)
     gram_finalize_wide_kernel(const PlanView v, double* out_gram) {
   __shared__ double t8[kWideWarps * tri(kMaxK)];
   __shared__ double G[kMaxK * kMaxK];
+  grid_wait();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t b = blockIdx.x;
   if (!header_ok(v)) return;
@@ -84,6 +87,7 @@ __global__ void __launch_bounds__(32 * kWideWarps)
 __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
     gram_finalize_kernel(const PlanView v, double* out_gram) {
   __shared__ double Gs[kSolveWarpsPerBlock][kMaxK * kMaxK];
+  grid_wait();
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int64_t b = (int64_t)blockIdx.x * kSolveWarpsPerBlock + wi;
   if (b >= v.n_buckets) return;
@@ -100,6 +104,8 @@ __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
 // result into the group's first row.  Each (row, entry) is read and written
 // by one thread only.
 __global__ void __launch_bounds__(256) group_reduce_kernel(const PlanView v) {
+  grid_wait();
+  grid_release();
   if (!header_ok(v)) return;
   const int P = tri(v.K);
   const int p = threadIdx.x;
@@ -134,13 +140,15 @@ cudaError_t launch_selftest_fp64(int op, const double* a, const double* b, doubl
   return cudaGetLastError();
 }
 
-cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s) {
+cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s, bool behind) {
   if (v.max_chunks <= kGroupMinChunks || v.b_hi <= v.b_lo) return cudaSuccess;
   const int64_t gx = (v.max_chunks + kGroupChunks - 1) / kGroupChunks;
   int64_t gy = v.b_hi - v.b_lo;
   if (gy > 65535) gy = 65535;
-  group_reduce_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, s>>>(v);
-  return cudaGetLastError();
+  PlanView va = v;
+  void* args[] = {&va};
+  return launch_behind((const void*)group_reduce_kernel, dim3((unsigned)gx, (unsigned)gy),
+                       dim3(256), args, 0, s, behind);
 }
 
 // Buckets of more chunks than this take a block each (below, a warp adds the
@@ -148,27 +156,31 @@ cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s) {
 constexpr int64_t kWideMinChunks = 32;
 
 cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_weights,
-                         int32_t* out_status, cudaStream_t s) {
+                         int32_t* out_status, cudaStream_t s, bool behind) {
   if (v.b_hi <= v.b_lo) return cudaSuccess;
-  if (v.max_chunks > kWideMinChunks) {
-    solve_wide_kernel<<<(unsigned)(v.b_hi - v.b_lo), 32 * kWideWarps, 0, s>>>(v, p, out_weights,
-                                                                             out_status);
-    return cudaGetLastError();
-  }
-  const int64_t grid = (v.b_hi - v.b_lo + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
-  solve_kernel<<<(unsigned)grid, 32 * kSolveWarpsPerBlock, 0, s>>>(v, p, out_weights, out_status);
-  return cudaGetLastError();
+  const int64_t nb = v.b_hi - v.b_lo;
+  const bool wide = v.max_chunks > kWideMinChunks;
+  const int64_t grid = wide ? nb : (nb + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
+  PlanView va = v;
+  SolveParams pa = p;
+  void* args[] = {&va, &pa, &out_weights, &out_status};
+  return launch_behind(wide ? (const void*)solve_wide_kernel : (const void*)solve_kernel,
+                       dim3((unsigned)grid),
+                       dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s, behind);
 }
 
-cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s) {
+cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s,
+                                 bool behind) {
   if (v.n_buckets == 0) return cudaSuccess;
-  if (v.max_chunks > kWideMinChunks) {
-    gram_finalize_wide_kernel<<<(unsigned)v.n_buckets, 32 * kWideWarps, 0, s>>>(v, out_gram);
-    return cudaGetLastError();
-  }
-  const int64_t grid = (v.n_buckets + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
-  gram_finalize_kernel<<<(unsigned)grid, 32 * kSolveWarpsPerBlock, 0, s>>>(v, out_gram);
-  return cudaGetLastError();
+  const bool wide = v.max_chunks > kWideMinChunks;
+  const int64_t grid =
+      wide ? v.n_buckets : (v.n_buckets + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
+  PlanView va = v;
+  void* args[] = {&va, &out_gram};
+  return launch_behind(wide ? (const void*)gram_finalize_wide_kernel
+                            : (const void*)gram_finalize_kernel,
+                       dim3((unsigned)grid),
+                       dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s, behind);
 }
 
 }  // namespace bkmoo
