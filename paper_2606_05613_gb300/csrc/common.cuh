@@ -344,6 +344,14 @@ const void* gram_prefetch_fn(int K, int dt);
 int gram_prefetch_smem(int K);
 int gram_prefetch_min_k();
 
+// Gram-pass kernels fed by bulk copies (same signature, gram_bulk_threads()
+// threads, gram_bulk_smem(K) bytes of dynamic shared memory), K = kBulkMinK ..
+// kBulkMaxK, nullptr outside; gram_bulk.cu.
+constexpr int kBulkMinK = 2, kBulkMaxK = 8;
+const void* gram_bulk_fn(int K, int dt);
+int gram_bulk_smem(int K);
+int gram_bulk_threads();
+
 // Combine kernels with a per-thread shared-memory prefetch (same signature,
 // combine_prefetch_smem(K) bytes of dynamic shared memory), every K;
 // combine_prefetch.cu, combine_prefetch_k9_16.cu.

@@ -266,14 +266,31 @@ int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool 
   // large K: the variant that prefetches into shared memory (gram_prefetch.cu)
   const bool pf = v.K >= gram_prefetch_min_k();
   const void* fn = pf ? gram_prefetch_fn(v.K, v.in_dtype) : gram_fn(v.K, v.in_dtype);
-  const int smem = pf ? gram_prefetch_smem(v.K) : 0;
-  int grid = 0;
-  if (persistent_grid(fn, kThreads, &grid, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
+  int smem = pf ? gram_prefetch_smem(v.K) : 0, threads = kThreads, grid = 0;
+  const void* bulk = gram_bulk_fn(v.K, v.in_dtype);
+  if (bulk) {
+    // Fed by bulk copies: with at most a chunk per SM, where a register
+    // kernel's CTA has too little in flight alone (64 chunks, K = 2..8: 1.04-1.3
+    // times as fast), and for K = 6 and 7, whose register kernels lose
+    // occupancy (3.2 GB: K = 6 bf16 512 -> 464 us, K = 7 fp32 481 -> 448; K = 2..5
+    // and 8 within 3 % either way).
+    int two = 0;   // two CTAs per SM
+    if (persistent_grid(bulk, gram_bulk_threads(), &two, gram_bulk_smem(v.K)) != cudaSuccess)
+      return BKMOO_ERR_CUDA;
+    if (2 * nch <= two || v.K == 6 || v.K == 7) {
+      fn = bulk;
+      smem = gram_bulk_smem(v.K);
+      threads = gram_bulk_threads();
+      grid = two;
+    }
+  }
+  if (fn != bulk && persistent_grid(fn, threads, &grid, smem) != cudaSuccess)
+    return BKMOO_ERR_CUDA;
   if (grid > nch) grid = (int)nch;
   GradPtrs ga = g;
   PlanView va = v;
   void* args[] = {&ga, &va};
-  if (cudaLaunchKernel(fn, dim3(grid), dim3(kThreads), args, smem, s) != cudaSuccess)
+  if (cudaLaunchKernel(fn, dim3(grid), dim3(threads), args, smem, s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
   if (launch_group_reduce(v, s, behind) != cudaSuccess) return BKMOO_ERR_CUDA;
   return BKMOO_OK;
@@ -283,16 +300,17 @@ int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_
                    cudaStream_t s) {
   const int64_t nch = v.c_hi - v.c_lo;
   if (nch <= 0) return BKMOO_OK;
-  // A window of a few chunks per CTA: last chunk first, out of L2 (GPT-2 small
-  // bucket by bucket, 90 MB each, 1331 -> 1250 us).
-  const void* fn = combine_fn(v.K, v.in_dtype, out_dtype);
-  int smem = 0, grid = 0;
-  if (persistent_grid(fn, kThreads, &grid) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (nch > 4 * (int64_t)grid) {
-    fn = combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
-    smem = combine_prefetch_smem(v.K);
-    if (persistent_grid(fn, kThreads, &grid, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
-  }
+  // A short window: last chunk first, out of L2 (GPT-2 small bucket by bucket,
+  // 90 MB each, 1331 -> 1250 us).  The 50-60 MB that L2 still holds repay the
+  // 2-7 % by which the other kernel streams faster up to several hundred MB
+  // (K = 12, 773 MB: 338 us against 333).
+  const double bytes = (double)nch * v.chunk_elems * v.K * elem_bytes(v.in_dtype);
+  const bool shortw = bytes <= 384.0 * 1024 * 1024;
+  const void* fn = shortw ? combine_fn(v.K, v.in_dtype, out_dtype)
+                          : combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
+  const int smem = shortw ? 0 : combine_prefetch_smem(v.K);
+  int grid = 0;
+  if (persistent_grid(fn, kThreads, &grid, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
   if (grid > nch) grid = (int)nch;
   PlanView va = v;
   GradPtrs ga = g;

@@ -55,6 +55,7 @@
 // lets its copies land and returns.
 #pragma once
 
+#include "bulk_copy.cuh"
 #include "combine_impl.cuh"
 #include "gram_impl.cuh"
 #include "solver.cuh"
@@ -95,80 +96,7 @@ __host__ __device__ constexpr int stream_smem_bytes(int K) {
   return stream_ring_bytes(K) + 128;
 }
 
-// ---- barriers, bulk copies, tensor memory -----------------------------------
-
-__device__ __forceinline__ uint32_t st_smem(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void bar_init(uint64_t* b, unsigned n) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(st_smem(b)), "r"(n) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(uint64_t* b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(st_smem(b)) : "memory");
-}
-__device__ __forceinline__ void bar_arrive_tx(uint64_t* b, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(st_smem(b)),
-               "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool bar_try(uint64_t* b, unsigned parity) {
-  uint32_t ok;
-  asm volatile(
-      "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; "
-      "selp.u32 %0, 1, 0, p; }"
-      : "=r"(ok)
-      : "r"(st_smem(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool bar_test(uint64_t* b, unsigned parity) {
-  uint32_t ok;
-  asm volatile(
-      "{ .reg .pred p; mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2; "
-      "selp.u32 %0, 1, 0, p; }"
-      : "=r"(ok)
-      : "r"(st_smem(b)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned bytes, uint64_t* bar,
-                                          uint64_t pol) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1], %2, [%3], %4;" ::"r"(st_smem(dst)),
-      "l"(src), "r"(bytes), "r"(st_smem(bar)), "l"(pol)
-      : "memory");
-}
-__device__ __forceinline__ uint64_t stream_policy(bool last) {
-  uint64_t p;
-  if (last) asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  else asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-// True on one lane of the (converged) warp.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{ .reg .pred p; elect.sync _|p, 0xffffffff; selp.u32 %0, 1, 0, p; }" : "=r"(p));
-  return p != 0;
-}
-__device__ __forceinline__ uint4 ld_shared_volatile(const uint4* p) {
-  uint4 x;
-  asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
-               : "r"(st_smem(p))
-               : "memory");
-  return x;
-}
-__device__ __forceinline__ void st_shared_volatile(uint4* p, const uint4& x) {
-  asm volatile("st.volatile.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(st_smem(p)), "r"(x.x),
-               "r"(x.y), "r"(x.z), "r"(x.w)
-               : "memory");
-}
-__device__ __forceinline__ uint64_t stream_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
+// ---- tensor memory -------------------------------------------------------------
 
 __device__ __forceinline__ void tmem_st4(uint32_t a, const uint4& x) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x.x),

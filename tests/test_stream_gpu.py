@@ -183,3 +183,26 @@ def test_stream_under_graph_capture():
         want = _run(res, grads, "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)[0]
         assert torch.equal(got, want)
         assert res.status() == 0
+
+
+@pytest.mark.parametrize("dt", [F32, BF16])
+@pytest.mark.parametrize("K", range(2, 9))
+def test_bulk_fed_gram_is_the_register_kernels(K, dt):
+    """Plans that take the bulk-fed Gram pass (few chunks; K = 6, 7 always)
+    against bkmoo_gram_noalloc, which runs the register kernels: the same
+    matrices bit for bit, at chunk, stage and vector edges."""
+    ch = 16384 if dt == F32 else 32768
+    plans = [[1, 5, 7, 8, 63, 4097, ch - 1, ch, ch + 1, 3 * ch + 9], [100 * ch + 3]]
+    if K in (6, 7):
+        plans.append([200 * ch, 301 * ch - 5, 17, 111 * ch + 1])
+    for sizes in plans:
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        grads = _grads(K, dt, int(off[-1]), K)
+        res = bk.Resolver(K, dt, off, DEV)
+        got = torch.zeros(len(sizes), K, K, dtype=torch.float64, device=DEV)
+        want = torch.zeros_like(got)
+        res.gram(grads, got)
+        bk.bkmoo_gram_noalloc(grads, off, want)
+        torch.cuda.synchronize()
+        assert res.status() == 0
+        assert torch.equal(got, want)
