@@ -375,6 +375,7 @@ const void* stream_fn_k7_8(int K, int dti);
 int stream_threads();
 int stream_smem(int K);
 int stream_stage_kib(int K);
+int stream_chunk_stages(int K);   // stages of a whole chunk
 
 // solve.cu
 // `behind`: launched behind the Gram pass (launch_behind).

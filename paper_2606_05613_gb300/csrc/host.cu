@@ -106,11 +106,13 @@ struct StreamShape {
   int n_stream, n_solve, team, lead_kib;
 };
 StreamShape stream_shape(const PlanView& v, int rule, int sms) {
-  // From a bucket's last partial to its coefficients on every SM, measured
-  // under load (us; globaltimer stamps, K = 2, 4, 8).
-  const int k = v.K <= 4 ? 0 : v.K - 4;
-  const double chain = rule == BKMOO_CAGRAD ? 16 + 6 * k
-                                            : (rule == BKMOO_PCGRAD ? 10 + 9 * k : 8 + 5.5 * k);
+  // From a bucket's last partial to its coefficients on every SM (us), from
+  // globaltimer stamps under load (K = 2, 4, 8) and, for K <= 4, the lead at
+  // which 1 and 4 MiB buckets run fastest.
+  const double k4 = v.K < 4 ? v.K : 4, more = v.K > 4 ? v.K - 4 : 0;
+  const double chain = rule == BKMOO_CAGRAD   ? 8 + 2 * k4 + 6 * more
+                       : rule == BKMOO_PCGRAD ? 1 + 2.25 * k4 + 9 * more
+                                              : 1.3 + 1.8 * k4 + 5.5 * more;
   const int64_t nb = v.b_hi - v.b_lo, nch = v.c_hi - v.c_lo;
   const int64_t sets = (v.max_chunks + kSetChunks - 1) / kSetChunks;
   StreamShape s;
@@ -130,12 +132,12 @@ StreamShape stream_shape(const PlanView& v, int rule, int sms) {
   s.n_stream = sms - s.n_solve;
   if (s.n_stream > nch) s.n_stream = (int)nch;
   // the copies in flight, a chunk, and what the Gram streams during the chain
-  // (25-35 KiB per SM and us); more lets the kept part of the window shrink
-  // (K = 4, 1 MiB fp32 buckets, MGDA: 500 KiB 0.92, 650 0.90, 800 0.95, 1300
-  // 1.06 us per bucket)
-  // and for buckets of more than a chunk per SM, which complete in waves of
-  // chunks, part of a chunk more (8 Qwen3-8B layers: 624 KiB 3353, 800 3291, 1200
-  // 3342 us)
+  // (about 30 KiB per SM and us).  Less and the Gram stands still for the
+  // chain, more and less of the window is kept (2.4 GB fp32 in 4 MiB buckets,
+  // MGDA, us: K = 2 at 350 KiB 547, 400 534, 496 573; K = 3 460 590, 510 529, 640
+  // 559; K = 4 570 559, 624 544), and for buckets of more than a chunk per SM,
+  // which complete in waves of chunks, part of a chunk more (8 Qwen3-8B layers,
+  // K = 4: 624 KiB 3353, 800 3288, 1200 3391)
   s.lead_kib = (int)(64 * v.K + 128 + 30 * chain);
   if (nch > nb * sms) s.lead_kib += 44 * v.K;
   return s;
@@ -167,7 +169,10 @@ int launch_stream(const GradPtrs& g, const PlanView& v, const SolveParams& sp, v
   const int kib = stream_stage_kib(v.K);
   sv.n_stream = sh.n_stream;
   sv.team = sh.team;
-  sv.lead = sh.lead_kib / kib;
+  // (never less than a chunk and a stage: the combination of a chunk starts
+  // after its Gram)
+  const int least = stream_chunk_stages(v.K) + 1;
+  sv.lead = sh.lead_kib / kib > least ? sh.lead_kib / kib : least;
   // 48-58 MB of L2 in all, what the re-read still finds there (K = 4, 1 MiB
   // buckets: 256 KiB per SM 871, 320 841, 384 818 us; more finds no more)
   sv.l2_stages = (v.K <= 4 ? 384 : 320) / kib;

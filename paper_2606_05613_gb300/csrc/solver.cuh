@@ -2117,9 +2117,10 @@ __device__ __forceinline__ bool solve_fast_k(int rule, const double* G, const fl
 // after the caller's __syncwarp).
 __device__ bool solve_fast(int K, int rule, const double* G, const float* Gf,
                            const SolveParams& p, int64_t b, int lane, double* beta_out) {
-  if (K >= 3 && (K <= 4   ? solve_pivot<4>(K, rule, G, Gf, p, lane, beta_out)
-                 : K <= 8 ? solve_pivot<8>(K, rule, G, Gf, p, lane, beta_out)
-                          : solve_pivot<kMaxK>(K, rule, G, Gf, p, lane, beta_out)))
+  if (K >= 3 && (rule == BKMOO_MGDA || rule == BKMOO_CAGRAD) &&
+      (K <= 4   ? solve_pivot<4>(K, rule, G, Gf, p, lane, beta_out)
+       : K <= 8 ? solve_pivot<8>(K, rule, G, Gf, p, lane, beta_out)
+                : solve_pivot<kMaxK>(K, rule, G, Gf, p, lane, beta_out)))
     return true;
   if (K > kEnumMaxK && rule != BKMOO_PCGRAD) return solve_large(K, rule, G, Gf, p, lane, beta_out);
   switch (K) {

@@ -12,4 +12,5 @@ const void* stream_fn_k1_2(int K, int dti) {
 int stream_threads() { return 32 * kStreamWarps; }
 int stream_smem(int K) { return stream_smem_bytes(K); }
 int stream_stage_kib(int K) { return stream_stage_bytes(K) / 1024; }
+int stream_chunk_stages(int K) { return kVecPerThread / stream_items(K); }
 }  // namespace bkmoo
