@@ -7,16 +7,16 @@
 // (2K + 1) e bytes per element with the output; here a chunk's vectors stay in
 // tensor memory (256 KB per SM that this path has no matrix product for) or
 // are asked to stay in L2 between their two uses, and only the rest is read
-// again.  Measured under ncu, GPT-2 small (K = 4 fp32, 25 MiB buckets): 3.43
-// GB of DRAM traffic for 1.99 GB of gradients (4.48 with two reads) at 6.5 TB/s;
-// 1 MiB buckets: 3.25 GB for 1.92 (4.32).  What is kept is set by the bytes in
-// flight between the two uses (a bucket, the solve's chain, the copy rings)
-// against 39 MB of tensor memory and about 50 MB of L2 (of 126 MB: a probe that
-// re-reads a stream D bytes later finds all of it up to D = 60 MB with
-// evict_last, 45 MB of it at D = 120 MB), so a shorter chain means fewer
-// bytes.  Time, three launches -> this kernel (us): GPT-2 small 672 -> 523,
-// 250 M fp32 elements K = 4 in 1 MiB buckets 1280 -> 839, 500 M K = 2 in 4 MiB
-// buckets 1274 (cluster-per-bucket kernel, since removed) -> 935.
+// again.  Measured under ncu, GPT-2 small (K = 4 fp32, 25 MiB buckets): 3.36
+// GB of DRAM traffic for 1.99 GB of gradients (4.48 with two reads) at 6.6 TB/s;
+// 120 M fp32 elements in 1 MiB buckets: 2.67 GB for 1.92 (4.32).  What is kept is
+// set by the bytes in flight between the two uses (a bucket, the solve's chain,
+// the copy rings) against 39 MB of tensor memory and about 55 MB of L2 (of 126
+// MB: a probe that re-reads a stream D bytes later finds all of it up to D = 60
+// MB with evict_last, 45 MB of it at D = 120 MB), so a shorter chain means fewer
+// bytes.  Time, before -> now (us): GPT-2 small 672 -> 520, 250 M fp32 elements
+// K = 4 in 1 MiB buckets 1279 -> 820 (three launches before), 500 M K = 2 in 4 MiB
+// buckets 1275 (a cluster-per-bucket kernel, since removed) -> 874.
 //
 // Chunks and arithmetic are those of the three launches: the same chunks, the
 // same thread for every vector, the same order of every sum, so the results
