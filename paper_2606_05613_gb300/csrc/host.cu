@@ -89,14 +89,18 @@ const void* stream_fn(int K, int dt) {
 // 10-20 us, small plans (K = 8, 4 Mi bf16 elements: 53 against 50) and buckets
 // under 1 MiB of gradients (K = 8 CAGrad, 2048 of 512 KiB: 409 against 425 us,
 // PCGrad 470 against 444), and with many buckets of which little stays on the
-// chip (K = 8, 134 buckets of 25 MiB bf16: 6.05 ms against 5.95).
+// chip (K = 8, 134 buckets of 25 MiB bf16: 6.05 ms against 5.95; one bucket of
+// 32 GB at K = 8 9.69 against 9.54, of 65.5 GB at K = 4 20.70 against 20.62; of
+// 16 GB at K = 4 5.04 against 5.10).
 bool stream_wins(const PlanView& v, const int64_t* off) {
   if (v.K > kStreamMaxK || v.c_hi <= v.c_lo) return false;
   const int64_t nb = v.b_hi - v.b_lo;
   const double bytes = (double)(off[v.b_hi] - off[v.b_lo]) * v.K * elem_bytes(v.in_dtype);
   const double mib = 1024.0 * 1024.0;
   if (v.K >= 5)
-    return bytes >= 96.0 * mib && bytes >= 1.0 * mib * nb && (nb <= 8 || bytes < 128.0 * mib * nb);
+    return bytes >= 96.0 * mib && bytes >= 1.0 * mib * nb &&
+           bytes < (nb <= 8 ? 1024.0 : 128.0) * mib * nb;
+  if (bytes >= 32768.0 * mib * nb) return false;
   return nb <= 64 || bytes >= 0.5 * mib * nb;
 }
 
