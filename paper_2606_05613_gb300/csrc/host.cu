@@ -314,7 +314,13 @@ int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_
   // 2-7 % by which the other kernel streams faster up to several hundred MB
   // (K = 12, 773 MB: 338 us against 333).
   const double bytes = (double)nch * v.chunk_elems * v.K * elem_bytes(v.in_dtype);
-  const bool shortw = bytes <= 384.0 * 1024 * 1024;
+  // Not with fewer chunks than SMs: there the prefetching kernel was the faster
+  // one (K = 8 bf16, 1.1 M elements, PCGrad, three launches: 46 us against 52).
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return BKMOO_ERR_CUDA;
+  const bool shortw = bytes <= 384.0 * 1024 * 1024 && nch > sms;
   const void* fn = shortw ? combine_fn(v.K, v.in_dtype, out_dtype)
                           : combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
   const int smem = shortw ? 0 : combine_prefetch_smem(v.K);
