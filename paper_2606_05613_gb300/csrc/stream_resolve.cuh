@@ -902,7 +902,11 @@ __global__ void __launch_bounds__(32 * kStreamWarps, 1)
   else if (wid == kP + 1) stream_rows<K>(
         sh, sv, n_own, blockIdx.x == 0 && (prm.flags & BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE), lane);
   else if (wid == kP + 2) stream_comb_producer<K, DT>(sh, cbuf, g, sv, n_own, lane);
+  // A Gram warp that gives up leaves its chunk's tensor-memory stores in
+  // flight; none may be when the memory is handed back.
   __syncwarp();
+  tmem_wait_st();
+  tmem_wait_ld();
   tmem_fence_before();
   __syncthreads();
   if (wid == kP + 1)

@@ -160,6 +160,26 @@ def test_stream_from_several_streams_and_threads(shared):
         _same(want, o)
 
 
+@pytest.mark.parametrize("withhold", [bk.BKMOO_FLAG_TEST_WITHHOLD,
+                                      bk.BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE])
+@pytest.mark.parametrize("K,dt", [(1, F32), (4, BF16), (8, F32)])
+def test_stream_gives_up_inside_a_chunk(K, dt, withhold):
+    """A wait that runs out while the other CTAs are several chunks into a
+    bucket (their Gram warps leave a chunk unfinished, its tensor-memory stores
+    in flight): the call ends with BKMOO_ERR_TIMEOUT, and the next one on the
+    same workspace, which takes the same tensor memory, is right."""
+    ch = 16384 if dt == F32 else 32768
+    off = np.array([0, 700 * ch, 1400 * ch + 5], dtype=np.int64)
+    grads = _grads(K, dt, int(off[-1]), K)
+    res = bk.Resolver(K, dt, off, DEV)
+    want = _run(res, grads, "mgda", dt, bk.BKMOO_FLAG_THREE_PASS)
+    _run(res, grads, "mgda", dt, bk.BKMOO_FLAG_FUSED | withhold)
+    assert res.status() == bk.BKMOO_ERR_TIMEOUT
+    got = _run(res, grads, "mgda", dt, bk.BKMOO_FLAG_FUSED)
+    assert res.status() == 0
+    _same(want, got)
+
+
 def test_stream_under_graph_capture():
     """Captured once, replayed on new inputs."""
     off = _plan(F32, "sets")
