@@ -47,7 +47,7 @@ def _args():
     ap.add_argument("--rule", default="mgda", choices=["mgda", "pcgrad", "cagrad", "mean"])
     ap.add_argument("--path", default="auto", choices=["auto", "fused", "3pass"],
                     help="auto: the library's per-plan choice; fused: one launch per step "
-                         "(re-read from L2); 3pass: Gram, solve and combination launches")
+                         "(K <= 8); 3pass: Gram, solve and combination launches")
     ap.add_argument("--hook", action="store_true",
                     help="time a synthetic training step of a GPT-2-small-shaped transformer "
                          "with the per-bucket resolve inside the backward pass (BucketMOO) "
@@ -173,18 +173,6 @@ class ClockSampler:
         reasons = sorted({n for r in rows for n, v in zip(names, r[5:9]) if v == "Active"})
         return {"sm_mhz": sm[len(sm) // 2] if sm else None, "sm_max_mhz": mx,
                 "reasons": reasons, "samples": len(rows)}
-
-
-def launches_per_step(w, off, fused):
-    """Kernels of this library one resolve launches: the streamed kernel; or
-    Gram pass, solve and combination, plus the group pre-reduction of the
-    chunk partials when a bucket has more than 1024 chunks."""
-    import numpy as np
-    if fused and w.K <= 8:
-        return 1
-    ch = 16384 if w.dtype == "f32" else 32768
-    longest = int(np.max(np.diff(np.asarray(off, dtype=np.int64))))
-    return 3 + (1 if (longest + ch - 1) // ch > 1024 else 0)
 
 
 def base_config(w, off, rule):
@@ -459,6 +447,9 @@ def main():
     elif a.path == "3pass":
         params.flags |= bk.BKMOO_FLAG_THREE_PASS
 
+    launches = bk.bkmoo_resolve_launches(
+        w.K, bk.BKMOO_F32 if tdt == torch.float32 else bk.BKMOO_BF16, a.rule, off, params)
+
     def step(evs=None):
         if evs is not None:
             arr = (ctypes.c_void_p * 4)(*[e.cuda_event for e in evs])
@@ -504,9 +495,7 @@ def main():
     peak, peak_kind = _peaks()
     e_in = w.elem_bytes
     e_out = out.element_size()
-    # one launch records the last three events together after it; a solve and
-    # a combination of their own take microseconds
-    fused = float(per[:, 1:].sum(axis=1).mean()) < 0.005
+    fused = launches == 1
     if fused:   # one launch: Gram + solve + combination
         kern = {"fused": (per[:, 0].mean(), (w.K * e_in + e_out) * N, "fused")}
         dom = "fused"
@@ -547,7 +536,7 @@ def main():
                           "frac_2k1_of_measured": step_bytes_2k1 / (ms_step * 1e-3) / GB / peak,
                           "frac_k1_of_measured": step_bytes_k1 / (ms_step * 1e-3) / GB / peak,
                           "frac_2k1_of_8tbs": step_bytes_2k1 / (ms_step * 1e-3) / GB / 8000.0},
-        "gpu_launches": launches_per_step(w, off, fused) * a.steps,
+        "gpu_launches": launches * a.steps,
         "clocks": clk,
         "bucket_status_counts": {str(k): int((st == k).sum()) for k in sorted(set(st.tolist()))},
         "host_wall_ms_per_step": 1e3 * wall / a.steps,

@@ -290,9 +290,10 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype,
  * elements of out_dir, the rows of out_weights / out_status and the
  * workspace partials of other buckets are not touched, so calls for disjoint
  * bucket ranges may run concurrently on different streams.  Results are
- * bit-identical to those of bkmoo_resolve for the same buckets; the path is
- * chosen as there.  The workspace
- * status word is not cleared (other calls may be in flight); device-side
+ * bit-identical to those of bkmoo_resolve for the same buckets.  Ranges of
+ * more than two buckets take one launch where bkmoo_resolve would for a plan of
+ * these buckets; one or two always three launches, which share the SMs with
+ * whatever runs beside them.  The workspace status word is not cleared (other calls may be in flight); device-side
  * errors are recorded into it.  BKMOO_FLAG_FUSED and p->events are ignored.
  */
 int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
@@ -359,20 +360,31 @@ int bkmoo_resolve_host(const void* const* host_grads, int32_t K, int32_t in_dtyp
 int bkmoo_workspace_status(const void* ws, void* stream, int32_t* status);
 
 /*
- * bkmoo_resolve_path -- what is certain of bkmoo_resolve's path for this
- * plan, rule and flags: *path = 1 or 2 for one launch (see BKMOO_FLAG_FUSED),
- * 0 where it may take the three launches.  (1 and 2 named two earlier one-launch
- * kernels and keep their conditions; the same kernel now runs for both.)
- * BKMOO_FLAG_THREE_PASS gives 0 (always three launches); BKMOO_FLAG_FUSED
- * gives 1 for K <= 4 (2 with BKMOO_FLAG_TEST_WITHHOLD), 2 for K = 5..8, 0
- * above.  Without either flag: 1 when K <= 2 and the plan has at most 8
- * buckets and 4 Mi elements per language, or when 2 <= K <= 4, the largest
- * bucket holds at least 2 MiB per language and its K gradients together at
- * most 12 MiB (and at least 6 MiB for bf16; for CAGrad fp32 only and at least
- * 8 MiB), and at least 90 % of the elements lie in buckets of at least half
- * the largest; 0 otherwise, where one launch runs for most plans of K <= 4 and
- * many of K = 5..8.  Host only; BKMOO_ERR_INVALID on bad arguments.
- * bkmoo_resolve_host always takes the three launches per window.
+ * bkmoo_resolve_launches -- the kernels that bkmoo_resolve launches for this
+ * plan, rule and *p (NULL: the defaults): *launches = 1 for the one launch (see
+ * BKMOO_FLAG_FUSED), 3 for Gram, solve and combination, 4 when a bucket has
+ * more than 1024 chunks and its partials are pre-reduced, 0 for no bucket.  (A
+ * device or context that cannot hold the one launch takes three where this
+ * says 1.)  Host only; BKMOO_ERR_INVALID on bad arguments.
+ * bkmoo_resolve_buckets decides by the same rule over its range, except that
+ * ranges of one or two buckets always take the three launches;
+ * bkmoo_resolve_host takes the three launches per window.
+ */
+int bkmoo_resolve_launches(int32_t K, int32_t in_dtype, int32_t rule, const int64_t* offsets,
+                           int64_t n_buckets, const bkmoo_params* p, int32_t* launches);
+
+/*
+ * bkmoo_resolve_path -- a classification of plans from two earlier one-launch
+ * kernels, kept with its answers for programs that record it.  It decides
+ * nothing and does not tell the path (bkmoo_resolve_launches does).
+ * BKMOO_FLAG_THREE_PASS gives 0; BKMOO_FLAG_FUSED gives 1 for K <= 4 (2 with
+ * BKMOO_FLAG_TEST_WITHHOLD), 2 for K = 5..8, 0 above.  Without either flag: 1
+ * when K <= 2 and the plan has at most 8 buckets and 4 Mi elements per
+ * language, or when 2 <= K <= 4, the largest bucket holds at least 2 MiB per
+ * language and its K gradients together at most 12 MiB (and at least 6 MiB for
+ * bf16; for CAGrad fp32 only and at least 8 MiB), and at least 90 % of the
+ * elements lie in buckets of at least half the largest; 0 otherwise.  Host
+ * only; BKMOO_ERR_INVALID on bad arguments.
  */
 int bkmoo_resolve_path(int32_t K, int32_t in_dtype, int32_t rule, const int64_t* offsets,
                        int64_t n_buckets, uint32_t flags, int32_t* path);

@@ -202,8 +202,15 @@ int launch_stream(const GradPtrs& g, const PlanView& v, const SolveParams& sp, v
   return BKMOO_OK;
 }
 
-// bkmoo_resolve_path's answer (see bkmoo.h): 1 or 2 where one launch is
-// certain, by the flags or for the plans listed there; 0 otherwise.
+// Whether a resolve of the view's window takes the streamed launch: the one
+// rule behind bkmoo_resolve, bkmoo_resolve_buckets and bkmoo_resolve_launches.
+bool streams(const PlanView& v, const int64_t* off, uint32_t flags) {
+  if (flags & BKMOO_FLAG_THREE_PASS) return false;
+  if (flags & BKMOO_FLAG_FUSED) return v.K <= kStreamMaxK && v.c_hi > v.c_lo;
+  return stream_wins(v, off);
+}
+
+// bkmoo_resolve_path's answer (see bkmoo.h); decides nothing.
 int choose_path(int32_t K, int32_t dt, int32_t rule, const int64_t* off, int64_t B,
                 uint32_t flags) {
   if (flags & BKMOO_FLAG_THREE_PASS) return 0;
@@ -227,6 +234,23 @@ int choose_path(int32_t K, int32_t dt, int32_t rule, const int64_t* off, int64_t
   return big * 10 >= off[B] * 9 ? 1 : 0;
 }
 
+// The part of a plan view that K, the dtype and the offsets give, as a window
+// over the whole plan.
+void plan_sizes(int32_t K, int32_t dt, const int64_t* offsets, int64_t B, PlanView* v) {
+  const int64_t ch = chunk_elems(dt);
+  v->K = K;
+  v->in_dtype = dt;
+  v->n_buckets = B;
+  v->n_chunks = count_chunks(offsets, B, ch);
+  v->chunk_elems = ch;
+  v->max_chunks = 0;
+  for (int64_t b = 0; b < B; ++b) {
+    const int64_t n = (offsets[b + 1] - offsets[b] + ch - 1) / ch;
+    if (n > v->max_chunks) v->max_chunks = n;
+  }
+  full_window(*v);
+}
+
 // Common checks of bkmoo_gram / bkmoo_resolve; fills the plan view.
 int prepare(const void* const* grads, int32_t K, int32_t dt, const int64_t* offsets,
             int64_t B, void* ws, size_t ws_bytes, PlanView* v, GradPtrs* g) {
@@ -235,9 +259,8 @@ int prepare(const void* const* grads, int32_t K, int32_t dt, const int64_t* offs
   if (!aligned(ws, 256)) return BKMOO_ERR_INVALID;
   for (int k = 0; k < K; ++k)
     if (!grads[k] || !aligned(grads[k], 16)) return BKMOO_ERR_INVALID;
-  const int64_t ch = chunk_elems(dt);
-  const int64_t nch = count_chunks(offsets, B, ch);
-  const WsLayout L = ws_layout(K, B, nch);
+  plan_sizes(K, dt, offsets, B, v);
+  const WsLayout L = ws_layout(K, B, v->n_chunks);
   if (ws_bytes < L.total_all) return BKMOO_ERR_WORKSPACE;
   char* base = static_cast<char*>(ws);
   v->hdr = reinterpret_cast<WsHeader*>(base);
@@ -245,18 +268,7 @@ int prepare(const void* const* grads, int32_t K, int32_t dt, const int64_t* offs
   v->chunk_prefix = reinterpret_cast<const int64_t*>(base + L.chunk_prefix);
   v->partials = reinterpret_cast<double*>(base + L.partials);
   v->beta = reinterpret_cast<float*>(base + L.beta);
-  v->n_buckets = B;
-  v->n_chunks = nch;
-  v->chunk_elems = ch;
   v->plan_hash = plan_hash(K, dt, offsets, B);
-  v->K = K;
-  v->in_dtype = dt;
-  v->max_chunks = 0;
-  for (int64_t b = 0; b < B; ++b) {
-    const int64_t n = (offsets[b + 1] - offsets[b] + ch - 1) / ch;
-    if (n > v->max_chunks) v->max_chunks = n;
-  }
-  full_window(*v);
   std::memset(g, 0, sizeof(*g));
   for (int k = 0; k < K; ++k) g->p[k] = grads[k];
   return BKMOO_OK;
@@ -541,8 +553,7 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype, const i
   cudaEvent_t* ev = static_cast<cudaEvent_t*>(prm.events);
   const SolveParams sp = solve_params(rule, prm);
   if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (choose_path(K, in_dtype, rule, offsets, n_buckets, prm.flags) != 0 ||
-      (!(prm.flags & BKMOO_FLAG_THREE_PASS) && stream_wins(v, offsets))) {
+  if (streams(v, offsets, prm.flags)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, true, &taken, s);
     if (r != BKMOO_OK) return r;
@@ -589,7 +600,7 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   // the caller overlaps them with; the streamed launch needs all of them at
   // once (a training step that resolves each bucket beside the backward pass:
   // 263.9 ms with three launches per bucket, 267.3 streamed).
-  if (!(prm.flags & BKMOO_FLAG_THREE_PASS) && b_hi - b_lo > 2 && stream_wins(v, offsets)) {
+  if (b_hi - b_lo > 2 && streams(v, offsets, prm.flags & ~BKMOO_FLAG_FUSED)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
     if (r != BKMOO_OK || taken) return r;
@@ -775,6 +786,24 @@ int bkmoo_resolve_path(int32_t K, int32_t in_dtype, int32_t rule, const int64_t*
       rule > BKMOO_MEAN || !offsets_ok(offsets, n_buckets))
     return BKMOO_ERR_INVALID;
   *path = choose_path(K, in_dtype, rule, offsets, n_buckets, flags);
+  return BKMOO_OK;
+}
+
+int bkmoo_resolve_launches(int32_t K, int32_t in_dtype, int32_t rule, const int64_t* offsets,
+                           int64_t n_buckets, const bkmoo_params* p, int32_t* launches) {
+  if (!launches || K < 1 || K > kMaxK || !dtype_ok(in_dtype) || rule < BKMOO_MGDA ||
+      rule > BKMOO_MEAN || !offsets_ok(offsets, n_buckets))
+    return BKMOO_ERR_INVALID;
+  bkmoo_params prm;
+  if (p) prm = *p;
+  else bkmoo_default_params(&prm);
+  if (!params_ok(prm)) return BKMOO_ERR_INVALID;
+  PlanView v;
+  std::memset(&v, 0, sizeof v);
+  plan_sizes(K, in_dtype, offsets, n_buckets, &v);
+  if (n_buckets == 0) *launches = 0;
+  else if (streams(v, offsets, prm.flags)) *launches = 1;
+  else *launches = v.max_chunks > kGroupMinChunks ? 4 : 3;
   return BKMOO_OK;
 }
 

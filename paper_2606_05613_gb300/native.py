@@ -108,6 +108,10 @@ def load():
         lib.bkmoo_resolve_path.restype = ctypes.c_int
         lib.bkmoo_resolve_path.argtypes = [i32, i32, i32, vp, i64, ctypes.c_uint32,
                                            ctypes.POINTER(ctypes.c_int32)]
+        lib.bkmoo_resolve_launches.restype = ctypes.c_int
+        lib.bkmoo_resolve_launches.argtypes = [i32, i32, i32, vp, i64,
+                                               ctypes.POINTER(bkmoo_params),
+                                               ctypes.POINTER(ctypes.c_int32)]
         lib.bkmoo_selftest_fp64.restype = ctypes.c_int
         lib.bkmoo_selftest_fp64.argtypes = [i32, vp, vp, vp, i64, vp]
         _lib = lib
@@ -296,9 +300,21 @@ def bkmoo_version() -> int:
     return int(load().bkmoo_version())
 
 
+def bkmoo_resolve_launches(K: int, in_dtype: int, rule, offsets, params=None) -> int:
+    """Kernels that bkmoo_resolve launches: 1 (the one launch), 3 or 4."""
+    if isinstance(rule, str):
+        rule = RULES[rule]
+    off = _offsets_array(offsets)
+    out = ctypes.c_int32(-1)
+    _check(load().bkmoo_resolve_launches(K, in_dtype, rule, off.ctypes.data, len(off) - 1,
+                                         ctypes.byref(params) if params is not None else None,
+                                         ctypes.byref(out)), "bkmoo_resolve_launches")
+    return int(out.value)
+
+
 def bkmoo_resolve_path(K: int, in_dtype: int, rule, offsets, flags: int) -> int:
-    """1 or 2: one launch; 0: bkmoo_resolve may take the three launches (see
-    include/bkmoo.h)."""
+    """A classification of plans kept from earlier kernels; the launches of a
+    call are bkmoo_resolve_launches' answer (see include/bkmoo.h)."""
     if isinstance(rule, str):
         rule = RULES[rule]
     off = _offsets_array(offsets)

@@ -405,3 +405,52 @@ def test_resolve_path_choice():
         4, F32, "mgda", sweep4, bk.BKMOO_FLAG_FUSED | bk.BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE) == 1
     with pytest.raises(bk.BkmooError):
         bk.bkmoo_resolve_path(0, F32, "mgda", sweep4, 0)
+
+
+def _params(flags=0, **kw):
+    p = bk.bkmoo_default_params()
+    p.flags |= flags
+    for k, v in kw.items():
+        setattr(p, k, v)
+    return p
+
+
+def test_resolve_launches_tells_the_rule_that_decides():
+    """The launches of bkmoo_resolve, plan by plan: the streamed launch for
+    nearly every plan of K <= 4 and some of K = 5..8, three launches elsewhere
+    (four with the pre-reduction of a bucket of more than 1024 chunks), as
+    measured; the flags force either."""
+    F32, BF16 = bk.BKMOO_F32, bk.BKMOO_BF16
+    MiB = inputs.MiB
+
+    def n(K, dt, off, rule="mgda", **kw):
+        return bk.bkmoo_resolve_launches(K, dt, rule, off, _params(**kw))
+
+    models = [(inputs.qwen3_8b_sizes(), 2, 4, BF16, 1), (inputs.gpt2_small_sizes(), 4, 4, F32, 1),
+              (inputs.llama32_1b_sizes(), 2, 8, BF16, 3)]
+    for sizes, eb, K, dt, want in models:
+        off = bk.bkmoo_plan(sizes, eb, 25 * MiB)
+        assert n(K, dt, off) == want
+        assert n(K, dt, off, flags=bk.BKMOO_FLAG_THREE_PASS) == 3
+        assert n(K, dt, off, flags=bk.BKMOO_FLAG_FUSED) == 1
+    for rule in ("mgda", "pcgrad", "cagrad", "mean"):
+        for K in (1, 2, 3, 4):
+            assert n(K, F32, bk.bkmoo_plan([10**9], 4, MiB), rule) == 1
+            assert n(K, F32, [0, 1, 5, 20000], rule) == 1
+    # many buckets of little: three launches, also where two larger ones make
+    # most of the plan
+    assert n(4, F32, np.arange(0, 300 * 16385, 16385, dtype=np.int64)) == 3
+    mixed = np.array([0, 600000, 1200000] + [1200000 + 300 * (i + 1) for i in range(200)],
+                     dtype=np.int64)
+    assert n(4, F32, mixed) == 3
+    assert n(2, F32, mixed) == 3
+    # a bucket of more than 1024 chunks (of 16384 fp32 elements)
+    assert n(16, F32, [0, 1024 * 16384]) == 3
+    assert n(16, F32, [0, 1024 * 16384 + 1]) == 4
+    assert n(16, F32, [0, 100], flags=bk.BKMOO_FLAG_FUSED) == 3   # K > 8: the flag is ignored
+    assert n(4, F32, [0]) == 0
+    for bad in [(0, F32, [0, 4]), (17, F32, [0, 4]), (4, 5, [0, 4]), (4, F32, [0, 4, 4])]:
+        with pytest.raises(bk.BkmooError):
+            n(*bad)
+    with pytest.raises(bk.BkmooError):
+        n(4, F32, [0, 4], max_iter=-1)
