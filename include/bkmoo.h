@@ -77,7 +77,11 @@ typedef enum { BKMOO_F32 = 0, BKMOO_BF16 = 1 } bkmoo_dtype;
                                           follows the Gram bucket by bucket
                                           while the gradients are still on
                                           the chip, for K <= 8; above, ignored
-                                          (three launches).  The results are
+                                          (three launches), and where a solve
+                                          may be long: MGDA (but for the K = 2
+                                          closed form) and CAGrad with max_iter
+                                          above 1024 or, for K >= 3, without
+                                          BKMOO_FLAG_POLISH.  The results are
                                           those of the three launches, bit for
                                           bit.  Without this flag the faster
                                           of the two is taken.              */

@@ -202,10 +202,27 @@ int launch_stream(const GradPtrs& g, const PlanView& v, const SolveParams& sp, v
   return BKMOO_OK;
 }
 
+// Whether a bucket's solve is short enough for the streamed launch, whose
+// solver warps are few and on which everything waits.  Frank-Wolfe is one lane's
+// fp64 steps, up to max_iter of them (K = 4: 0.9 us a step for MGDA, 2 for
+// CAGrad; K = 8: 5 and 13).  Without POLISH every bucket of K >= 3 runs it: 32
+// buckets of 25 MiB bf16, K = 4, 256 steps, streamed 4.3 ms (CAGrad 7.9), three
+// launches, which solve all buckets at once, 1.3 (1.5).  (K = 2 is exact after
+// one line search: 434 us streamed, 639 three.)  With POLISH only buckets whose
+// exact solution is not certified do; 1024 steps are 13 ms, far from the 2 s
+// after which a wait gives up.
+constexpr int32_t kStreamMaxIter = 1024;
+bool solve_is_short(int32_t K, int32_t rule, const bkmoo_params& p) {
+  if (K == 1 || rule == BKMOO_PCGRAD || rule == BKMOO_MEAN) return true;
+  if (K == 2 && rule == BKMOO_MGDA && (p.flags & BKMOO_FLAG_CLOSED_FORM_K2)) return true;
+  return p.max_iter <= kStreamMaxIter && (K == 2 || (p.flags & BKMOO_FLAG_POLISH));
+}
+
 // Whether a resolve of the view's window takes the streamed launch: the one
 // rule behind bkmoo_resolve, bkmoo_resolve_buckets and bkmoo_resolve_launches.
-bool streams(const PlanView& v, const int64_t* off, uint32_t flags) {
-  if (flags & BKMOO_FLAG_THREE_PASS) return false;
+bool streams(const PlanView& v, const int64_t* off, int32_t rule, const bkmoo_params& p,
+             uint32_t flags) {
+  if ((flags & BKMOO_FLAG_THREE_PASS) || !solve_is_short(v.K, rule, p)) return false;
   if (flags & BKMOO_FLAG_FUSED) return v.K <= kStreamMaxK && v.c_hi > v.c_lo;
   return stream_wins(v, off);
 }
@@ -553,7 +570,7 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype, const i
   cudaEvent_t* ev = static_cast<cudaEvent_t*>(prm.events);
   const SolveParams sp = solve_params(rule, prm);
   if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (streams(v, offsets, prm.flags)) {
+  if (streams(v, offsets, rule, prm, prm.flags)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, true, &taken, s);
     if (r != BKMOO_OK) return r;
@@ -600,7 +617,7 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   // the caller overlaps them with; the streamed launch needs all of them at
   // once (a training step that resolves each bucket beside the backward pass:
   // 263.9 ms with three launches per bucket, 267.3 streamed).
-  if (b_hi - b_lo > 2 && streams(v, offsets, prm.flags & ~BKMOO_FLAG_FUSED)) {
+  if (b_hi - b_lo > 2 && streams(v, offsets, rule, prm, prm.flags & ~BKMOO_FLAG_FUSED)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
     if (r != BKMOO_OK || taken) return r;
@@ -802,7 +819,7 @@ int bkmoo_resolve_launches(int32_t K, int32_t in_dtype, int32_t rule, const int6
   std::memset(&v, 0, sizeof v);
   plan_sizes(K, in_dtype, offsets, n_buckets, &v);
   if (n_buckets == 0) *launches = 0;
-  else if (streams(v, offsets, prm.flags)) *launches = 1;
+  else if (streams(v, offsets, rule, prm, prm.flags)) *launches = 1;
   else *launches = v.max_chunks > kGroupMinChunks ? 4 : 3;
   return BKMOO_OK;
 }

@@ -444,6 +444,25 @@ def test_resolve_launches_tells_the_rule_that_decides():
                      dtype=np.int64)
     assert n(4, F32, mixed) == 3
     assert n(2, F32, mixed) == 3
+    # rules that iterate: K >= 3 without the exact completion, and caps that a
+    # bounded wait could not cover, with and without the flag that asks for one
+    # launch; the K = 2 closed form, PCGrad and the mean never iterate
+    sweep = bk.bkmoo_plan([10**9], 4, MiB)
+    for f in (0, bk.BKMOO_FLAG_FUSED):
+        for rule in ("mgda", "cagrad"):
+            p = bk.bkmoo_default_params()
+            p.flags = f
+            for K, want in ((1, 1), (2, 1), (3, 3), (4, 3), (8, 3)):
+                assert bk.bkmoo_resolve_launches(K, F32, rule, sweep, p) == want, (f, rule, K)
+            for K in (3, 4):
+                assert n(K, F32, sweep, rule, flags=f, max_iter=1024) == 1
+                assert n(K, F32, sweep, rule, flags=f, max_iter=1025) == 3
+        assert n(2, F32, sweep, "mgda", flags=f, max_iter=10**9) == 1
+        assert n(2, F32, sweep, "cagrad", flags=f, max_iter=10**9) == 3
+        for rule in ("pcgrad", "mean"):
+            p = bk.bkmoo_default_params()
+            p.flags, p.max_iter = f, 10**9
+            assert bk.bkmoo_resolve_launches(4, F32, rule, sweep, p) == 1
     # a bucket of more than 1024 chunks (of 16384 fp32 elements)
     assert n(16, F32, [0, 1024 * 16384]) == 3
     assert n(16, F32, [0, 1024 * 16384 + 1]) == 4

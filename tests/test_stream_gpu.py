@@ -180,6 +180,29 @@ def test_stream_gives_up_inside_a_chunk(K, dt, withhold):
     _same(want, got)
 
 
+@pytest.mark.parametrize("rule", ["mgda", "cagrad"])
+@pytest.mark.parametrize("K", [2, 3, 4])
+def test_frank_wolfe_alone_is_the_three_launches(K, rule):
+    """Without the exact completion the default call (three launches for
+    K >= 3, whatever BKMOO_FLAG_FUSED says) gives the three launches' bits."""
+    off = _plan(F32, "sets")
+    grads = _grads(K, F32, int(off[-1]), 17)
+    res = bk.Resolver(K, F32, off, DEV)
+    got = []
+    for flag in (bk.BKMOO_FLAG_THREE_PASS, 0, bk.BKMOO_FLAG_FUSED):
+        p = bk.bkmoo_default_params()
+        p.flags = flag
+        out = torch.zeros(int(off[-1]), device=DEV)
+        w = torch.zeros(res.n_buckets, K, device=DEV)
+        st = torch.zeros(res.n_buckets, dtype=torch.int32, device=DEV)
+        res.resolve(grads, rule, out, params=p, out_weights=w, out_status=st)
+        torch.cuda.synchronize()
+        assert res.status() == 0
+        got.append((out, w, st))
+    _same(got[0], got[1])
+    _same(got[0], got[2])
+
+
 def test_stream_under_graph_capture():
     """Captured once, replayed on new inputs."""
     off = _plan(F32, "sets")
