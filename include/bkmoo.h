@@ -87,21 +87,22 @@ typedef enum { BKMOO_F32 = 0, BKMOO_BF16 = 1 } bkmoo_dtype;
                                           of the two is taken.              */
 #define BKMOO_FLAG_THREE_PASS 0x8u     /* always the three-launch path (Gram,
                                           solve, combination)               */
-#define BKMOO_FLAG_TEST_WITHHOLD 0x100u /* testing failure detection, where
-                                          the one launch runs: it never
-                                          publishes its first bucket's
-                                          coefficients, so its bounded waits
-                                          (about 2 s) run out and the call
-                                          ends with BKMOO_ERR_TIMEOUT in the
+#define BKMOO_FLAG_TEST_WITHHOLD 0x100u /* testing failure detection, with
+                                          BKMOO_FLAG_FUSED only, where the one
+                                          launch runs: it never publishes its
+                                          first bucket's coefficients, so its
+                                          bounded waits (about 2 s) run out and
+                                          the call ends with BKMOO_ERR_TIMEOUT in the
                                           workspace status word; the output
                                           is then undefined                 */
 #define BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE 0x200u /* testing failure detection,
-                                          where the one launch runs: its first
-                                          CTA never publishes its first
-                                          chunk's partial Gram, so the bounded
-                                          wait for it (about 2 s) runs out,
-                                          every other wait ends at once, and
-                                          the call ends with
+                                          with BKMOO_FLAG_FUSED only, where the
+                                          one launch runs: its first CTA never
+                                          publishes its first chunk's partial
+                                          Gram, so the bounded wait for it
+                                          (about 2 s) runs out, every other
+                                          wait ends at once, and the call ends
+                                          with
                                           BKMOO_ERR_TIMEOUT in the workspace
                                           status word; the output is then
                                           undefined                         */

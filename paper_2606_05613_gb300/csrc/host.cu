@@ -369,15 +369,19 @@ bool params_ok(const bkmoo_params& p) {
   return p.max_iter >= 0 && p.cagrad_c >= 0.0 && p.cagrad_c < 1.0 && p.tol >= 0.0;
 }
 
-SolveParams solve_params(int32_t rule, const bkmoo_params& prm) {
+// `flags`: those of prm that count for the call; the withholding test flags only
+// with BKMOO_FLAG_FUSED.
+SolveParams solve_params(int32_t rule, const bkmoo_params& prm, uint32_t flags) {
   SolveParams sp;
+  if (!(flags & BKMOO_FLAG_FUSED))
+    flags &= ~(BKMOO_FLAG_TEST_WITHHOLD | BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE);
   sp.rule = rule;
   sp.max_iter = prm.max_iter;
   sp.tol = prm.tol;
   sp.cagrad_c = prm.cagrad_c;
   sp.seed = prm.seed;
   sp.step = prm.step;
-  sp.flags = prm.flags;
+  sp.flags = flags;
   return sp;
 }
 
@@ -568,7 +572,7 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype, const i
   if (r != BKMOO_OK) return r;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaEvent_t* ev = static_cast<cudaEvent_t*>(prm.events);
-  const SolveParams sp = solve_params(rule, prm);
+  const SolveParams sp = solve_params(rule, prm, prm.flags);
   if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return BKMOO_ERR_CUDA;
   if (streams(v, offsets, rule, prm, prm.flags)) {
     bool taken = false;
@@ -612,12 +616,13 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   for (int64_t b = b_lo; b < b_hi; ++b) c += (offsets[b + 1] - offsets[b] + v.chunk_elems - 1) / v.chunk_elems;
   v.c_hi = c;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const SolveParams sp = solve_params(rule, prm);
+  const uint32_t flags = prm.flags & ~BKMOO_FLAG_FUSED;
+  const SolveParams sp = solve_params(rule, prm, flags);
   // One or two buckets: the three launches, which share the SMs with whatever
   // the caller overlaps them with; the streamed launch needs all of them at
   // once (a training step that resolves each bucket beside the backward pass:
   // 263.9 ms with three launches per bucket, 267.3 streamed).
-  if (b_hi - b_lo > 2 && streams(v, offsets, rule, prm, prm.flags & ~BKMOO_FLAG_FUSED)) {
+  if (b_hi - b_lo > 2 && streams(v, offsets, rule, prm, flags)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
     if (r != BKMOO_OK || taken) return r;
@@ -675,7 +680,7 @@ int bkmoo_resolve_host(const void* const* host_grads, int32_t K, int32_t in_dtyp
   if (cudaMemsetAsync(&v.hdr->status, 0, sizeof(int32_t), s) != cudaSuccess)
     return BKMOO_ERR_CUDA;
   if (n_buckets == 0) return BKMOO_OK;
-  const SolveParams sp = solve_params(rule, prm);
+  const SolveParams sp = solve_params(rule, prm, prm.flags);
 
   // Slot layout: K input regions then the output region, each of
   // region_bytes(cap) bytes.

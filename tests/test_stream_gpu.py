@@ -180,6 +180,20 @@ def test_stream_gives_up_inside_a_chunk(K, dt, withhold):
     _same(want, got)
 
 
+@pytest.mark.parametrize("step", [0, 3])
+def test_withholding_flags_need_the_fused_flag(step):
+    """A default call, and one over ranges (which ignores BKMOO_FLAG_FUSED), is
+    right whatever the withholding test flags say."""
+    off = _plan(F32, "sets")
+    grads = _grads(4, F32, int(off[-1]), 2)
+    res = bk.Resolver(4, F32, off, DEV)
+    want = _run(res, grads, "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)
+    flag = bk.BKMOO_FLAG_TEST_WITHHOLD | bk.BKMOO_FLAG_TEST_WITHHOLD_EXCHANGE
+    got = _run(res, grads, "mgda", F32, flag | (bk.BKMOO_FLAG_FUSED if step else 0), step=step)
+    assert res.status() == 0
+    _same(want, got)
+
+
 @pytest.mark.parametrize("rule", ["mgda", "cagrad"])
 @pytest.mark.parametrize("K", [2, 3, 4])
 def test_frank_wolfe_alone_is_the_three_launches(K, rule):
