@@ -243,14 +243,15 @@ __device__ __forceinline__ double sum_rows8(const double* src, int64_t rs, int64
   return tree8(t);
 }
 // A set: the first kSetChunks (or all left) of `left` rows, a whole one in
-// one round trip.
+// one round trip.  (No partial is -0, so adding the first eight to 0, as
+// sum_rows8 does, would change nothing.)
 __device__ __forceinline__ double set_sum(const double* row, int64_t rs, int64_t left) {
   if (left < kSetChunks) return sum_rows8(row, rs, left);
   double x[kSetChunks], u[8];
 #pragma unroll
   for (int i = 0; i < kSetChunks; ++i) x[i] = row[i * rs];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) u[i] = (0.0 + x[i]) + x[i + 8];
+  for (int i = 0; i < 8; ++i) u[i] = x[i] + x[i + 8];
   return tree8(u);
 }
 // Chunk rows: for K <= kStreamMaxK sets of kSetChunks rows, then the sets'

@@ -84,18 +84,14 @@ __device__ void reduce_bucket(const PlanView& v, int64_t b, double* G, int lane)
   __syncwarp();
 }
 
-// The same by a block of eight warps, for buckets of many chunks: warp w forms
-// the interleaved sum w of every entry (t8: [8][P] in shared memory), which
-// the caller adds by tree8_entry once the block has synchronised.
+// n rows (rs doubles apart) by a block of eight warps: warp w forms the
+// interleaved sum w of every entry (t8: [8][P] in shared memory); tree8_entry
+// adds them once the block has synchronised.  `sets`: the rows are chunk rows
+// of K <= kStreamMaxK (sum_chunk_rows), else flat (sum_rows8).
 constexpr int kWideWarps = 8;
-__device__ void reduce_bucket_wide(const PlanView& v, int64_t b, double* t8, int lane, int w) {
-  const int K = v.K, P = tri(K);
-  const int64_t c0 = v.chunk_prefix[b], n0 = v.chunk_prefix[b + 1] - c0;
-  const bool pre = n0 > kGroupMinChunks;
-  const int64_t n = pre ? (n0 + kGroupChunks - 1) / kGroupChunks : n0;
-  const int64_t rs = pre ? kGroupChunks * P : P;
-  const double* src = v.partials + c0 * P;
-  if (K <= kStreamMaxK && !pre) {
+__device__ void sum_rows_wide(const double* src, int64_t rs, int64_t n, int P, bool sets,
+                              double* t8, int lane, int w) {
+  if (sets) {
     for (int p = lane; p < P; p += 32) {
       double t = 0.0;
       for (int64_t at = (int64_t)w * kSetChunks; at < n; at += kWideWarps * kSetChunks)
@@ -127,13 +123,27 @@ __device__ void reduce_bucket_wide(const PlanView& v, int64_t b, double* t8, int
   for (int e = 0; e < E; ++e)
     if (lane + 32 * e < P) t8[w * P + lane + 32 * e] = t[e];
 }
+__device__ __forceinline__ double tree8_entry(const double* t8, int P, int p) {
+  const double* t = t8 + p;
+  return ((t[0] + t[P]) + (t[2 * P] + t[3 * P])) +
+         ((t[4 * P] + t[5 * P]) + (t[6 * P] + t[7 * P]));
+}
+// reduce_bucket by a block of eight warps, for buckets of many chunks; the
+// caller takes G from the sums (gram_from_sums) once the block has
+// synchronised.
+__device__ void reduce_bucket_wide(const PlanView& v, int64_t b, double* t8, int lane, int w) {
+  const int K = v.K, P = tri(K);
+  const int64_t c0 = v.chunk_prefix[b], n = v.chunk_prefix[b + 1] - c0;
+  const bool pre = n > kGroupMinChunks;
+  sum_rows_wide(v.partials + c0 * P, pre ? kGroupChunks * P : P,
+                pre ? (n + kGroupChunks - 1) / kGroupChunks : n, P, K <= kStreamMaxK && !pre, t8,
+                lane, w);
+}
 // One warp: G from the eight interleaved sums.
 __device__ void gram_from_sums(int K, const double* t8, double* G, int lane) {
   const int P = tri(K);
   for (int p = lane; p < P; p += 32) {
-    const double* t = t8 + p;
-    const double s = ((t[0] + t[P]) + (t[2 * P] + t[3 * P])) +
-                     ((t[4 * P] + t[5 * P]) + (t[6 * P] + t[7 * P]));
+    const double s = tree8_entry(t8, P, p);
     int i = 0, r = p;
     while (r >= K - i) {
       r -= K - i;

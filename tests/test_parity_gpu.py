@@ -326,6 +326,34 @@ def test_huge_buckets_group_reduction(dt):
         _check_against_oracle(w, rule, off, hv, out, beta.cpu().numpy(), status.cpu().numpy(), dt)
 
 
+@pytest.mark.parametrize("K", [1, 4, 9, 16])
+def test_group_sums_beside_many_small_buckets(K):
+    """Buckets of more than 1024 chunks at the front, in the middle and at the
+    end of 11,000 small ones (several look-over rounds of the pre-reduction's
+    blocks): their Gram matrices are those of each alone, bit for bit."""
+    ch = 16384
+    small = [8] * 5500
+    sizes = [1025 * ch + 8] + small + [1024 * ch + 8] + small + [1030 * ch]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    n = int(off[-1])
+    gen = torch.Generator(device=DEV).manual_seed(K)
+    grads = [torch.randn(n, generator=gen, device=DEV) for _ in range(K)]
+    G = torch.zeros(len(sizes), K, K, dtype=torch.float64, device=DEV)
+    res = bk.Resolver(K, torch.float32, off, DEV)
+    res.gram(grads, G)
+    for b in (0, 1, 5501, 5502, len(sizes) - 1):
+        lo, hi = int(off[b]), int(off[b + 1])
+        part = [g[lo:hi] for g in grads]
+        alone = torch.zeros(1, K, K, dtype=torch.float64, device=DEV)
+        bk.Resolver(K, torch.float32, np.array([0, hi - lo]), DEV).gram(part, alone)
+        assert torch.equal(alone[0], G[b]), b
+        X = torch.stack([p.double() for p in part])
+        d = torch.linalg.vector_norm(X, dim=1)
+        # fp32 products and sums of at most 133 terms before the fp64 sums
+        assert ((alone[0] - X @ X.T).abs() <= 1e-5 * d[:, None] * d[None, :]).all()
+    assert res.status() == 0
+
+
 # ---------------------------------------------------------------------------
 # fused path (BKMOO_FLAG_FUSED): one persistent launch per resolve
 # ---------------------------------------------------------------------------
