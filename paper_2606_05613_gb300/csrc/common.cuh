@@ -378,6 +378,9 @@ int stream_smem(int K);
 int stream_stage_kib(int K);
 int stream_chunk_stages(int K);   // stages of a whole chunk
 
+// SMs of the current device (cached; host.cu).
+cudaError_t sm_count(int* n);
+
 // solve.cu
 // `behind`: launched behind the Gram pass (launch_behind).
 cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_weights,

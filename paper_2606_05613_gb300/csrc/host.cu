@@ -34,6 +34,18 @@ LaunchCache& cache() {
   return c;
 }
 
+// With the cache's lock held.
+cudaError_t device_sms(LaunchCache& c, int dev, int* n) {
+  auto it = c.sms.find(dev);
+  if (it == c.sms.end()) {
+    const cudaError_t e = cudaDeviceGetAttribute(n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    it = c.sms.emplace(dev, *n).first;
+  }
+  *n = it->second;
+  return cudaSuccess;
+}
+
 // Resident CTAs of `fn` on the current device times its SM count.  A kernel
 // with dynamic shared memory gets its limit raised to that size once (the
 // default limit of 48 KiB counts static and dynamic shared memory together).
@@ -43,13 +55,9 @@ cudaError_t persistent_grid(const void* fn, int threads, int* grid, int dyn_smem
   if (e != cudaSuccess) return e;
   LaunchCache& c = cache();
   std::lock_guard<std::mutex> lk(c.mu);
-  auto it = c.sms.find(dev);
-  if (it == c.sms.end()) {
-    int n = 0;
-    e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    it = c.sms.emplace(dev, n).first;
-  }
+  int sms = 0;
+  e = device_sms(c, dev, &sms);
+  if (e != cudaSuccess) return e;
   auto key = std::make_pair(dev, fn);
   auto jt = c.occ.find(key);
   if (jt == c.occ.end()) {
@@ -62,7 +70,7 @@ cudaError_t persistent_grid(const void* fn, int threads, int* grid, int dyn_smem
     if (e != cudaSuccess) return e;
     jt = c.occ.emplace(key, n < 1 ? 1 : n).first;
   }
-  *grid = it->second * jt->second;
+  *grid = sms * jt->second;
   return cudaSuccess;
 }
 
@@ -345,10 +353,8 @@ int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_
   const double bytes = (double)nch * v.chunk_elems * v.K * elem_bytes(v.in_dtype);
   // Not with fewer chunks than SMs: there the prefetching kernel was the faster
   // one (K = 8 bf16, 1.1 M elements, PCGrad, three launches: 46 us against 52).
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return BKMOO_ERR_CUDA;
+  int sms = 0;
+  if (sm_count(&sms) != cudaSuccess) return BKMOO_ERR_CUDA;
   const bool shortw = bytes <= 384.0 * 1024 * 1024 && nch > sms;
   const void* fn = shortw ? combine_fn(v.K, v.in_dtype, out_dtype)
                           : combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
@@ -442,6 +448,15 @@ int64_t slot_capacity(int32_t K, int32_t dti, int32_t dto, size_t bytes) {
 }
 
 }  // namespace
+
+cudaError_t bkmoo::sm_count(int* n) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  LaunchCache& c = cache();
+  std::lock_guard<std::mutex> lk(c.mu);
+  return device_sms(c, dev, n);
+}
 
 extern "C" {
 

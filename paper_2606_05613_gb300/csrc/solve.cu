@@ -1,7 +1,8 @@
-// Solve pass: one warp per bucket.  The warp reduces the bucket's per-chunk
-// Gram partials in a fixed order (lane p owns entry p of the triangle and adds
-// the chunks in ascending order, in fp64) into G in shared memory, then solves
-// the bucket's rule (solver.cuh) and writes beta and the bucket's status.
+// Solve pass: one warp, or one block of eight, per bucket.  It reduces the
+// bucket's per-chunk Gram partials in a fixed order (fp64; sum_chunk_rows in
+// common.cuh: sets of sixteen rows for K <= 8, eight interleaved sums) into G in
+// shared memory; one warp solves the bucket's rule (solver.cuh) and writes beta
+// and the bucket's status.
 #include "solver.cuh"
 
 namespace bkmoo {
@@ -36,10 +37,9 @@ __global__ void __launch_bounds__(32 * kSolveWarpsPerBlock)
   if (lane == 0 && out_status) out_status[b] = st;
 }
 
-// One block of eight warps per bucket, for plans with buckets of many chunks:
-// the rows of a bucket are then the longest part of the pass (one warp adds
-// them at one fp64 instruction per 64 cycles; a 400-chunk K = 4 bucket: 68 -> 60
-// us for the three launches of the bucket alone).
+// One block of eight warps per bucket (solve_wide, below): the warps share the
+// rows, one solves.  One warp adds rows at one fp64 instruction per 64 cycles; a
+// 400-chunk K = 4 bucket: 68 -> 60 us for the three launches of the bucket alone.
 __global__ void __launch_bounds__(32 * kWideWarps)
     solve_wide_kernel(const PlanView v, const SolveParams p, float* out_weights,
                       int32_t* out_status) {
@@ -166,36 +166,57 @@ cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s, bool behind) 
                        dim3(32 * kWideWarps), args, 0, s, behind);
 }
 
-// Buckets of more chunks than this take a block each (below, a warp adds the
-// rows in the time that the block's hand-off takes).
-constexpr int64_t kWideMinChunks = 32;
+// Whether a window's buckets take a block of eight warps each; otherwise a warp
+// each, four to a block, in a plain launch.  Launched behind the Gram pass, the
+// four-warp blocks gather on the few SMs that finish first and share their fp64
+// units: 608 buckets, K = 4, Frank-Wolfe alone 631 us behind, 293 plain, 489 with
+// a block a bucket; CAGrad, small buckets: 45, 35, 40.  A block a bucket, behind,
+// wins up to two buckets per SM (304, CAGrad: 28 against 42 and 31) and, by 0.04
+// us for each row of the longest bucket against 0.02 for each bucket, where that
+// bucket is long (1000 buckets of 300 elements beside one of 1000 chunks, K = 4:
+// 169 against 182, 2000 beside one of 400 147 against 116).
+static cudaError_t solve_wide(const PlanView& v, int64_t nb, bool* wide) {
+  int sms = 0;
+  const cudaError_t e = sm_count(&sms);
+  const int64_t rows = v.max_chunks > kGroupMinChunks
+                           ? (v.max_chunks + kGroupChunks - 1) / kGroupChunks
+                           : v.max_chunks;
+  *wide = nb <= 2 * (int64_t)sms || 2 * rows >= nb;
+  return e;
+}
 
 cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_weights,
                          int32_t* out_status, cudaStream_t s, bool behind) {
-  if (v.b_hi <= v.b_lo) return cudaSuccess;
   const int64_t nb = v.b_hi - v.b_lo;
-  const bool wide = v.max_chunks > kWideMinChunks;
+  if (nb <= 0) return cudaSuccess;
+  bool wide = false;
+  const cudaError_t e = solve_wide(v, nb, &wide);
+  if (e != cudaSuccess) return e;
   const int64_t grid = wide ? nb : (nb + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
   PlanView va = v;
   SolveParams pa = p;
   void* args[] = {&va, &pa, &out_weights, &out_status};
   return launch_behind(wide ? (const void*)solve_wide_kernel : (const void*)solve_kernel,
                        dim3((unsigned)grid),
-                       dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s, behind);
+                       dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s,
+                       behind && wide);
 }
 
 cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s,
                                  bool behind) {
-  if (v.n_buckets == 0) return cudaSuccess;
-  const bool wide = v.max_chunks > kWideMinChunks;
-  const int64_t grid =
-      wide ? v.n_buckets : (v.n_buckets + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
+  const int64_t nb = v.n_buckets;
+  if (nb == 0) return cudaSuccess;
+  bool wide = false;
+  const cudaError_t e = solve_wide(v, nb, &wide);
+  if (e != cudaSuccess) return e;
+  const int64_t grid = wide ? nb : (nb + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
   PlanView va = v;
   void* args[] = {&va, &out_gram};
   return launch_behind(wide ? (const void*)gram_finalize_wide_kernel
                             : (const void*)gram_finalize_kernel,
                        dim3((unsigned)grid),
-                       dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s, behind);
+                       dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s,
+                       behind && wide);
 }
 
 }  // namespace bkmoo

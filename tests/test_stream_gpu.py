@@ -263,3 +263,28 @@ def test_bulk_fed_gram_is_the_register_kernels(K, dt):
         torch.cuda.synchronize()
         assert res.status() == 0
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("K", [2, 8, 12])
+def test_solve_pass_at_the_edges_of_its_two_kernels(K):
+    """Plans on both sides of the lines between a block and a warp per bucket
+    (two buckets per SM; the longest bucket against the number of buckets),
+    three launches: weights and directions are those of each bucket resolved
+    alone, bit for bit."""
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+    ch = 16384
+    for sizes in ([64] * (2 * sms), [64] * (2 * sms + 1), [64] * (4 * sms) + [2 * sms * ch],
+                  [64] * (4 * sms) + [(2 * sms + 1) * ch]):
+        if K > 8 and len(sizes) > 2 * sms + 1:
+            continue                                     # 8 GB, and no other code
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        grads = _grads(K, F32, int(off[-1]), K)
+        res = bk.Resolver(K, F32, off, DEV)
+        out, w, st = _run(res, grads, "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)
+        torch.cuda.synchronize()
+        assert res.status() == 0 and not st.any()
+        for b in (0, 1, len(sizes) // 2, len(sizes) - 1):
+            lo, hi = int(off[b]), int(off[b + 1])
+            one = bk.Resolver(K, F32, np.array([0, hi - lo]), DEV)
+            alone = _run(one, [g[lo:hi] for g in grads], "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)
+            assert torch.equal(alone[1][0], w[b]) and torch.equal(alone[0], out[lo:hi])
