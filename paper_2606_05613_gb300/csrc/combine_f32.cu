@@ -1,9 +1,10 @@
-// Combination kernels for fp32 gradients, K = 1..16, fp32 or bf16 output.
+// Combination kernels that take the last chunk first, fp32 gradients, K = 1..4,
+// fp32 or bf16 output.
 #include "combine_impl.cuh"
 
 namespace bkmoo {
-namespace {
-BKMOO_COMBINE_TABLE(BKMOO_F32);
-}
+static const void* const kCombineTable[combine_last_first_max_k(BKMOO_F32)][2] = {
+    BKMOO_COMBINE_ROW(1, BKMOO_F32), BKMOO_COMBINE_ROW(2, BKMOO_F32),
+    BKMOO_COMBINE_ROW(3, BKMOO_F32), BKMOO_COMBINE_ROW(4, BKMOO_F32)};
 const void* combine_fn_f32(int K, int dtype_out) { return kCombineTable[K - 1][dtype_out]; }
 }  // namespace bkmoo

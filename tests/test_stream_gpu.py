@@ -288,3 +288,24 @@ def test_solve_pass_at_the_edges_of_its_two_kernels(K):
             one = bk.Resolver(K, F32, np.array([0, hi - lo]), DEV)
             alone = _run(one, [g[lo:hi] for g in grads], "mgda", F32, bk.BKMOO_FLAG_THREE_PASS)
             assert torch.equal(alone[1][0], w[b]) and torch.equal(alone[0], out[lo:hi])
+
+
+@pytest.mark.parametrize("dt", [F32, BF16])
+@pytest.mark.parametrize("K", [1, 2, 3, 4, 5])
+def test_combination_kernels_at_the_edges_of_their_rule(K, dt):
+    """Windows of as many chunks as SMs and one more, and the most chunks whose
+    gradients are 384 MiB and one more: the combination of the three launches
+    (last chunk first up to K = 4 fp32 and K = 3 bf16) writes the streamed
+    launch's bits, fp32 and bf16 out, in place too."""
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+    ch = 16384 if dt == F32 else 32768
+    most = (384 << 20) // (K * 262144)
+    for n in (sms, sms + 1, most, most + 1):
+        sizes = [ch + 9] * 3 + [(n - 8) * ch - 5] + [7, 2]       # n chunks, starts off the grid
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        grads = _grads(K, dt, int(off[-1]), n)
+        res = bk.Resolver(K, dt, off, DEV)
+        for odt, inplace in ((F32, False), (BF16, False), (dt, True)):
+            _same(_run(res, grads, "mgda", odt, bk.BKMOO_FLAG_THREE_PASS, inplace),
+                  _run(res, grads, "mgda", odt, bk.BKMOO_FLAG_FUSED, inplace))
+        assert res.status() == 0
