@@ -87,19 +87,32 @@ const void* stream_fn(int K, int dt) {
 }
 
 // Whether the streamed launch is the faster one for a window (both give the
-// same results).  Measured on GB300 against the three launches, K = 2, 4, 5
-// and 8, fp32 and bf16, MGDA, PCGrad and CAGrad, 2^18 to 2^28 elements in
-// buckets of 64 KiB to 100 MiB: it reads the gradients little more than once
-// and is 1.05-2.6 times as fast wherever the SMs' time goes into streaming.
-// It loses where it goes into solves, which it does on the few SMs it sets
-// aside: many buckets of less than 512 KiB of gradients (K = 4 CAGrad, 256
-// buckets of 64 KiB fp32: 61 us against 41), and for K >= 5, whose solves take
-// 10-20 us, small plans (K = 8, 4 Mi bf16 elements: 53 against 50) and buckets
-// under 1 MiB of gradients (K = 8 CAGrad, 2048 of 512 KiB: 409 against 425 us,
-// PCGrad 470 against 444), and with many buckets of which little stays on the
-// chip (K = 8, 134 buckets of 25 MiB bf16: 6.05 ms against 5.95; one bucket of
-// 32 GB at K = 8 9.69 against 9.54, of 65.5 GB at K = 4 20.70 against 20.62; of
-// 16 GB at K = 4 5.04 against 5.10).
+// same results).  Measured on GB300 against the three launches on inputs not in
+// L2 before: K = 1..8 fp32 and 2, 4, 5, 6, 8 bf16, MGDA, PCGrad and CAGrad, 1 to
+// 4096 equal buckets of 16 KiB to 100 MiB a language, up to 3.3 GB of gradients.
+// It reads the gradients little more than once and wins wherever the SMs' time
+// goes into streaming; it loses where it goes into solves, which it does on the
+// few SMs it sets aside.  Where it is taken it is at most 5 % behind, mostly 1.1
+// to 1.6 times as fast.  The lines (streamed / three, us, fp32):
+//  - K <= 4, more than 64 buckets: 0.5 MiB of gradients a bucket.  K = 4, 4096 of
+//    0.5 MiB MGDA 445 / 724, CAGrad 535 / 754; 4096 of 0.25 MiB 248 / 386, but CAGrad
+//    452 / 417; 1024 of 64 KiB 69 / 47, 129 / 55.  64 buckets of 64 KiB, CAGrad:
+//    26 / 25.
+//  - K >= 5, whose solves take 10-20 us: 96 MiB in all.  K = 8, 8 buckets of 4 MiB
+//    MGDA 38.5 / 35.6, PCGrad 52.6 / 46.2; 16 of 4 MiB 40.2 / 47.2, 54.5 / 59.6; 64
+//    of 2 MiB 54.6 / 66.8, 68.2 / 78.1.
+//  - K >= 5: 1 MiB a bucket.  K = 8, 256 of 0.5 MiB MGDA 65.7 / 69.7, PCGrad 106 /
+//    80; 128 of 1 MiB 54.9 / 68.3, 81.8 / 79.3; 256 of 1 MiB 84 / 113, 105 / 123.
+//  - K >= 5, little of a bucket stays on the chip: more than 8 buckets only below
+//    128 MiB each.  K = 5, 16 of 125 MiB MGDA 603 / 672, CAGrad 658 / 684; K = 6, 16
+//    of 150 MiB 743 / 799, 812 / 813; K = 8 bf16, 16 of 200 MiB 974 / 1037, 1049 /
+//    1049 (1100 / 1060 with an opposed language), 134 of 200 MiB 5967 / 5909; 8
+//    of 200 MiB 489 / 534, 519 / 547.
+//  - enormous buckets, of which nearly everything is read twice (ms): K >= 3 from
+//    1 GiB each (K = 4 0.8 GiB 4.96 / 4.98, 1.6 GiB 5.01 / 4.98, 4 GB 5.10 / 5.04, one
+//    of 65.5 GB 20.66 / 20.61; K = 3 1.2 GiB 3.91 / 3.87; K = 5 1 GiB 2.47 / 2.46; K = 8
+//    0.8 GiB 1.89 / 1.92, one of 20 GB 6.15 / 5.92); K <= 2, whose second read costs
+//    less, from 32 GiB (K = 2 4 GB 2.81 / 2.90; K = 1 the same within 1 %).
 bool stream_wins(const PlanView& v, const int64_t* off) {
   if (v.K > kStreamMaxK || v.c_hi <= v.c_lo) return false;
   const int64_t nb = v.b_hi - v.b_lo;
@@ -108,7 +121,7 @@ bool stream_wins(const PlanView& v, const int64_t* off) {
   if (v.K >= 5)
     return bytes >= 96.0 * mib && bytes >= 1.0 * mib * nb &&
            bytes < (nb <= 8 ? 1024.0 : 128.0) * mib * nb;
-  if (bytes >= 32768.0 * mib * nb) return false;
+  if (bytes >= (v.K <= 2 ? 32768.0 : 1024.0) * mib * nb) return false;
   return nb <= 64 || bytes >= 0.5 * mib * nb;
 }
 

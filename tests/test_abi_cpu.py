@@ -463,6 +463,17 @@ def test_resolve_launches_tells_the_rule_that_decides():
             p = bk.bkmoo_default_params()
             p.flags, p.max_iter = f, 10**9
             assert bk.bkmoo_resolve_launches(4, F32, rule, sweep, p) == 1
+    # both sides of the lines on sizes, 4 bytes an element
+    def even(nb, mib):
+        return np.arange(nb + 1, dtype=np.int64) * int(mib * MiB / 4)
+
+    for K, nb, mib, want in [(4, 64, 1 / 64, 1), (4, 65, 1 / 64, 3), (4, 65, 1 / 8, 1),
+                             (2, 1000, 1 / 4, 1), (2, 1000, 1 / 4 - 1 / 1024, 3),
+                             (8, 24, 1 / 2, 1), (8, 23, 1 / 2, 3), (8, 768, 1 / 8, 1),
+                             (8, 1000, 1 / 8 - 1 / 1024, 3), (8, 9, 16, 3), (8, 9, 16 - 1 / 64, 1),
+                             (8, 8, 128 - 1 / 64, 1), (8, 8, 128, 4), (4, 3, 256 - 1 / 64, 1),
+                             (4, 3, 256, 4), (2, 3, 256, 1), (2, 1, 1 << 14, 4)]:
+        assert n(K, F32, even(nb, mib)) == want, (K, nb, mib)
     # a bucket of more than 1024 chunks (of 16384 fp32 elements)
     assert n(16, F32, [0, 1024 * 16384]) == 3
     assert n(16, F32, [0, 1024 * 16384 + 1]) == 4
