@@ -209,13 +209,13 @@ int bkmoo_conflicts(const double* gram, int32_t K, int64_t n_buckets, float* out
  * device memory all belongs to the framework's caching allocator, or a C
  * caller in a process where another component owns device allocation.
  *
- * Same arguments, results and determinism as bkmoo_gram (the same kernels
- * run).  The scratch (bucket table and per-chunk partial sums) lives in a
+ * Same arguments, results (bit for bit) and determinism as bkmoo_gram.  The
+ * scratch (bucket table and per-chunk partial sums) lives in a
  * static device array of BKMOO_NOALLOC_SCRATCH_BYTES that every GPU which
  * loads this library keeps until the process exits; the bucket table reaches
  * it through kernel parameters, so no copy or allocating call is made.
  * Limits: at most BKMOO_NOALLOC_MAX_BUCKETS buckets and a problem whose
- * workspace (bkmoo_workspace_size) fits the array -- about 13 billion
+ * bucket table and partial sums fit the array -- about 13 billion
  * elements per language for K = 4 and 1 billion for K = 16 with bf16
  * gradients (half as many with fp32); larger problems return
  * BKMOO_ERR_WORKSPACE.
@@ -271,9 +271,15 @@ int bkmoo_gram_noalloc(const void* const* grads, int32_t K, int32_t in_dtype,
  *   K, in_dtype and offsets.
  * Path: three launches (Gram, solve, combination) or one launch that does the
  *   same bucket by bucket (see BKMOO_FLAG_FUSED), whichever is faster for the
- *   plan and rule; the results are the same bit for bit and deterministic.
- *   The one launch is cooperative (every CTA resident at once); on a device
- *   or context that cannot hold it the three launches run.
+ *   plan and rule (bkmoo_resolve_launches tells); the results are the same bit
+ *   for bit and deterministic.  The one launch is cooperative: it starts once
+ *   every SM is free and holds them all until it ends, so work on other streams
+ *   runs before or after it, not beside it; on a device or context that cannot
+ *   hold it the three launches run.  Its CTAs wait for one another, at most 2 s
+ *   at a time: a wait that runs out ends the call with BKMOO_ERR_TIMEOUT in the
+ *   workspace status word and out_dir partly written (in place: that gradient).
+ *   With BKMOO_FLAG_THREE_PASS neither holds: the launches share the GPU, and
+ *   no CTA waits for another.
  * Returns BKMOO_OK once the work is queued on `stream`.
  */
 int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype,

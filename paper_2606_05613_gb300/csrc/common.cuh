@@ -256,7 +256,7 @@ __device__ __forceinline__ double set_sum(const double* row, int64_t rs, int64_t
 }
 // Chunk rows: for K <= kStreamMaxK sets of kSetChunks rows, then the sets'
 // sums in the same way -- the order in which the streamed kernel, whose sets
-// are summed by different CTAs, arrives at them.
+// are summed by different warps of a team, arrives at them.
 __device__ __forceinline__ double sum_chunk_rows(const double* src, int64_t rs, int64_t n, int K) {
   if (K > kStreamMaxK) return sum_rows8(src, rs, n);
   double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};

@@ -170,7 +170,8 @@ extern "C" int bkmoo_gram_noalloc(const void* const* grads, int32_t K, int32_t i
   std::memset(&g, 0, sizeof g);
   for (int k = 0; k < K; ++k) g.p[k] = grads[k];
 
-  // the same Gram-pass kernel as bkmoo_gram (the prefetching variant for large K)
+  // the register kernels, or the prefetching one for large K: the partials of
+  // bkmoo_gram, which feeds some plans by bulk copies instead, bit for bit
   const bool pf = K >= gram_prefetch_min_k();
   const void* fn = pf ? gram_prefetch_fn(K, in_dtype)
                       : (in_dtype == BKMOO_F32 ? gram_partials_fn_f32(K) : gram_partials_fn_bf16(K));

@@ -6,13 +6,14 @@
 //
 //  MGDA (Eq. 3; bucket form Eq. 6 over the simplex of Algorithm 1):
 //    K = 2 (flag CLOSED_FORM_K2): gamma = clamp(<g2 - g1, g2> / ||g1 - g2||^2, 0, 1).
-//    2 <= K <= 5 with POLISH: exact, by enumeration of the supports, one per
-//      lane: lane l takes S = the bits of l + 1, finds the affine
-//      minimum-norm point of S in fp32 and keeps it if it lies in the
-//      simplex; the least norm wins, is refined in fp64 and checked.
-//    K >= 6 with POLISH: Wolfe's minimum-norm-point algorithm in fp32 with a
-//      lane-parallel Gauss-Jordan, one fp64 refinement of the final support
-//      and the same check.
+//    With POLISH, exact: for K >= 3 block pivoting from the full support (fp32
+//      LU, refined and checked in fp64; solve_pivot).  What that does not
+//      settle: K <= 5 by enumeration of the supports, one per lane: lane l takes
+//      S = the bits of l + 1, finds the affine minimum-norm point of S in fp32
+//      and keeps it if it lies in the simplex; the least norm wins, is refined
+//      in fp64 and checked.  K >= 6 by Wolfe's minimum-norm-point algorithm in
+//      fp32 with a lane-parallel Gauss-Jordan, one fp64 refinement of the final
+//      support and the same check.
 //    Without POLISH, or when a check fails: Frank-Wolfe from the best pair
 //      with exact line search (lane 0, fp64), then (POLISH) an exact
 //      active-set completion in the manner of Wolfe's minimum-norm-point
@@ -22,12 +23,11 @@
 //      while some g_j has <d, g_j> < ||d||^2.
 //  CAGrad (Eq. 4; Eq. 7): the dual min_{w in simplex} F(w),
 //    F(w) = <g0, g_w> + c ||g0|| ||g_w||, beta = 1/K + c ||g0|| w / ||g_w||.
-//    K <= 5 with POLISH: exact, one support per lane, with the closed-form
-//      stationary point of F on the support's affine hull (fp32 search,
-//      fp64 refinement and check).
-//    K >= 6 with POLISH: the same kind of active-set method in fp32 with the
-//      lane-parallel Gauss-Jordan, from the best vertex; fp64 refinement and
-//      check.
+//    With POLISH, exact: for K >= 3 block pivoting as above.  What that does not
+//      settle: K <= 5 one support per lane, with the closed-form stationary point
+//      of F on the support's affine hull (fp32 search, fp64 refinement and
+//      check); K >= 6 the same kind of active-set method as for MGDA, from the
+//      best vertex.
 //    Without POLISH, or when a check fails: Frank-Wolfe with exact line
 //      search from the best vertex (lane 0, fp64), then (POLISH) the same
 //      kind of active-set completion.
@@ -57,10 +57,11 @@ constexpr double kPivot = 1e-13;   // smallest pivot of a non-singular system
 // partial reduction
 // ---------------------------------------------------------------------------
 
-// Lane p sums entry p of the bucket's chunk partials in a fixed order: eight
-// interleaved fp64 running sums (chunk c0 + 8m + j goes to sum j), added by a
-// fixed tree; eight independent chains hide the fp64 add latency, which a
-// single chain pays once per chunk (1600 chunks in a 100 MiB fp32 bucket).
+// Lane p sums entry p of the bucket's chunk partials in a fixed order
+// (sum_chunk_rows): eight interleaved fp64 sums, added by a fixed tree, of sets
+// of sixteen rows (K <= 8) or of the rows; the independent chains hide the fp64
+// add latency, which a single chain pays once per chunk (1600 chunks in a
+// 100 MiB fp32 bucket).
 // A bucket of more than kGroupMinChunks chunks was pre-reduced by
 // group_reduce_kernel: its group sums sit in the rows of the first chunk of
 // each group of kGroupChunks, and those rows are what is summed here.

@@ -14,9 +14,8 @@
 // the copy rings) against 39 MB of tensor memory and about 55 MB of L2 (of 126
 // MB: a probe that re-reads a stream D bytes later finds all of it up to D = 60
 // MB with evict_last, 45 MB of it at D = 120 MB), so a shorter chain means fewer
-// bytes.  Time, before -> now (us): GPT-2 small 672 -> 520, 250 M fp32 elements
-// K = 4 in 1 MiB buckets 1279 -> 820 (three launches before), 500 M K = 2 in 4 MiB
-// buckets 1275 (a cluster-per-bucket kernel, since removed) -> 874.
+// bytes.  Three launches against this one (us): GPT-2 small 672, 520; 250 M fp32
+// elements K = 4 in 1 MiB buckets 1279, 820; 500 M K = 2 in 4 MiB buckets 1470, 874.
 //
 // Chunks and arithmetic are those of the three launches: the same chunks, the
 // same thread for every vector, the same order of every sum, so the results
@@ -185,7 +184,7 @@ constexpr int kStreamDesc = 32;     // Gram chunk descriptors in flight
 constexpr int kStreamRed = 3;       // chunks whose triangles await the row warp
 constexpr int kStreamLq = 128;      // stages with an L2 claim in flight
 
-constexpr int kStreamSolveWarps = 16;   // of a solver CTA
+constexpr int kStreamSolveWarps = kStreamWarps;   // of a solver CTA: all of them
 
 // A solver team's state (dynamic shared memory of a solver CTA).
 template <int K>
@@ -606,7 +605,7 @@ __device__ bool stream_set(StreamShared<K>& sh, const StreamView& sv, const uint
   return got;
 }
 
-// Solver CTAs: teams of sv.team warps (1, 2, 4 or 8), each with every
+// Solver CTAs: teams of sv.team warps (2, 4 or 8), each with every
 // n_teams-th bucket.  Warp q of a team sums the sets q, q + team, ... as their
 // rows arrive and adds set j's sums to the team's eight interleaved sums; the
 // team's first warp adds those, solves and publishes.  (The order is that of
@@ -619,7 +618,6 @@ __device__ void stream_solver_cta(StreamShared<K>& sh, unsigned char* dyn, const
   constexpr int P = tri(K), R = stream_row_words(K);
   const PlanView& v = sv.v;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (wid >= kStreamSolveWarps) return;
   const int tw = sv.team, team = wid / tw, q = wid - team * tw;
   const int per_cta = kStreamSolveWarps / tw;
   const int64_t n_teams = (int64_t)per_cta * (gridDim.x - sv.n_stream);
@@ -715,8 +713,8 @@ __device__ __forceinline__ void stream_combine_vec(const uint4 (&r)[K], const fl
   else store_out<BKMOO_BF16>(out, el, y, EPV);
 }
 
-// Combination warps: thread t has the vector positions of Gram thread t (of
-// the Gram threads t and t + 128 when there are four warps).
+// Combination warps: thread t has the vector positions of the Gram threads t and
+// t + 128.
 template <int K, int DT>
 __device__ void stream_combine(StreamShared<K>& sh, const unsigned char* cbuf, const GradPtrs& g,
                                const StreamView& sv, void* out, int dto, int n_own) {
@@ -727,8 +725,9 @@ __device__ void stream_combine(StreamShared<K>& sh, const unsigned char* cbuf, c
   constexpr int TS = stream_tmem_slots(K);
   constexpr int CT = 32 * kStreamCombWarps;
   static_assert(HV % CT == 0, "a half stage is whole positions of every combination thread");
+  static_assert(kThreads == 2 * CT, "two Gram threads' positions per combination thread");
   const int ct = threadIdx.x - kThreads, lane = ct & 31, c = ct >> 5;
-  const uint32_t tm = sh.tmem + ((uint32_t)(c & 3) << 21) + (CT == kThreads ? (uint32_t)(c >> 2) * 256u : 0u);
+  const uint32_t tm = sh.tmem + ((uint32_t)c << 21);
   uint32_t seq = 0;
   int slot = 0, th = 0;
   unsigned par = 0;
@@ -774,16 +773,15 @@ __device__ void stream_combine(StreamShared<K>& sh, const unsigned char* cbuf, c
       const bool held = sh.tseq[th] == seq;
       if (held) {
         tmem_fence_after();
-        // column halves: Gram warps 0-3 and 4-7; warp c has its own half, or
-        // both when there are four
-        constexpr int N = U * kThreads / CT;
+        // warp c reads both column halves: those of Gram warps c and c + 4
+        constexpr int N = 2 * U;
         uint4 r[N][K];
 #pragma unroll
         for (int u = 0; u < N; ++u)
 #pragma unroll
           for (int k = 0; k < K; ++k)
-            tmem_ld4(tm + (CT == kThreads ? 0u : (uint32_t)(u & 1) * 256u) +
-                         (uint32_t)(th * (K * U * 4) + (u * CT / kThreads * K + k) * 4),
+            tmem_ld4(tm + (uint32_t)(u & 1) * 256u +
+                         (uint32_t)(th * (K * U * 4) + (u / 2 * K + k) * 4),
                      r[u][k]);
         tmem_wait_ld();
         tmem_fence_before();
