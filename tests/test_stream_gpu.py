@@ -294,12 +294,12 @@ def test_solve_pass_at_the_edges_of_its_two_kernels(K):
 @pytest.mark.parametrize("K", [1, 2, 3, 4, 5])
 def test_combination_kernels_at_the_edges_of_their_rule(K, dt):
     """Windows of as many chunks as SMs and one more, and the most chunks whose
-    gradients are 384 MiB and one more: the combination of the three launches
+    gradients are 192 MiB and one more: the combination of the three launches
     (last chunk first up to K = 4 fp32 and K = 3 bf16) writes the streamed
     launch's bits, fp32 and bf16 out, in place too."""
     sms = torch.cuda.get_device_properties(DEV).multi_processor_count
     ch = 16384 if dt == F32 else 32768
-    most = (384 << 20) // (K * 262144)
+    most = (192 << 20) // (K * 65536)
     for n in (sms, sms + 1, most, most + 1):
         sizes = [ch + 9] * 3 + [(n - 8) * ch - 5] + [7, 2]       # n chunks, starts off the grid
         off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
