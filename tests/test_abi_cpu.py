@@ -338,11 +338,11 @@ def test_selftest_fp64_rejects_bad_arguments_without_launch():
 
 
 def test_resolve_path_choice():
-    """The per-plan path rule (measured on GB300): the cluster-per-bucket
-    fused kernel for K = 2..4 with buckets of at least 2 MiB whose K
+    """bkmoo_resolve_path's classification, kept from earlier kernels (it does
+    not decide): 1 for K = 2..4 with buckets of at least 2 MiB whose K
     gradients take at most 12 MiB (bf16: 6..12 MiB; CAGrad: fp32 and at
-    least 8 MiB), and for tiny plans; the three launches otherwise; the
-    flags force either path."""
+    least 8 MiB), and for tiny plans; 0 otherwise; the flags give their own
+    answers."""
     F32, BF16 = bk.BKMOO_F32, bk.BKMOO_BF16
     MiB = inputs.MiB
 
@@ -380,7 +380,7 @@ def test_resolve_path_choice():
     assert bk.bkmoo_resolve_path(2, F32, "cagrad", plan(1 << 21, MiB, 4), 0) == 1
     assert bk.bkmoo_resolve_path(2, F32, "mgda", plan(1 << 23, MiB, 4), 0) == 0
     assert bk.bkmoo_resolve_path(4, F32, "mgda", plan(1 << 20, MiB, 4), 0) == 0
-    # the benchmark's model workloads keep the three launches
+    # the benchmark's model workloads
     for sizes, eb, K, dt in [(inputs.qwen3_8b_sizes(), 2, 4, BF16),
                              (inputs.gpt2_small_sizes(), 4, 4, F32),
                              (inputs.llama32_1b_sizes(), 2, 8, BF16)]:

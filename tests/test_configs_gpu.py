@@ -131,8 +131,7 @@ def test_qwen3_8b_k4_bf16_mgda_cagrad():
     for fused in (False, True):
         for rule in ("mgda", "cagrad"):
             p = bk.bkmoo_default_params()
-            if fused:
-                p.flags |= bk.BKMOO_FLAG_FUSED
+            p.flags |= bk.BKMOO_FLAG_FUSED if fused else bk.BKMOO_FLAG_THREE_PASS
             res, out, beta, st = _resolve(w, off, grads, rule, p, res=res)
             assert (st == 0).all(), np.unique(st, return_counts=True)
             runs.append(Run("qwen-%s-%s" % (rule, "fused" if fused else "3pass"), off, rule, out,

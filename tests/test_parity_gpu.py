@@ -355,7 +355,7 @@ def test_group_sums_beside_many_small_buckets(K):
 
 
 # ---------------------------------------------------------------------------
-# fused path (BKMOO_FLAG_FUSED): one persistent launch per resolve
+# one launch per resolve (BKMOO_FLAG_FUSED; K > 8: three launches)
 # ---------------------------------------------------------------------------
 
 def _fused_params(seed=0, step=0, flags=None):
@@ -375,8 +375,7 @@ def test_fused_resolve_parity(rule, dt, out_dt, K):
 
 
 def test_fused_tiny_buckets_and_empty_slices():
-    """Buckets far smaller than the grid (most slices empty) and every
-    head / tail length."""
+    """Buckets far smaller than the grid and every head / tail length."""
     sizes = [1, 2, 3, 4, 5, 6, 7, 8, 9, 15, 16, 17, 31, 33, 1000, 8191, 8193, 300001]
     for dt in ("f32", "bf16"):
         w = _workload(3, dt, sizes, 400000)
@@ -405,21 +404,20 @@ def test_fused_deterministic_and_matches_three_pass():
     res.resolve(grads, "mgda", out_f, params=_fused_params())
     torch.cuda.synchronize()
     assert torch.equal(o1, out_f)                     # run to run
-    _, _, out_3, beta_3, _, _ = _run(w, "mgda", "f32")
-    np.testing.assert_allclose(beta_f, beta_3, atol=1e-5)
-    d3 = out_3.cpu().numpy().astype(np.float64)
-    df = o1.cpu().numpy().astype(np.float64)
-    assert np.linalg.norm(df - d3) <= 1e-5 * np.linalg.norm(d3)
+    p3 = bk.bkmoo_default_params()
+    p3.flags |= bk.BKMOO_FLAG_THREE_PASS
+    _, _, out_3, beta_3, _, _ = _run(w, "mgda", "f32", params=p3)
+    np.testing.assert_array_equal(beta_f, beta_3)     # path to path
+    assert torch.equal(o1, out_3)
 
 
 @pytest.mark.parametrize("rule", ["mgda", "pcgrad", "cagrad", "mean"])
 @pytest.mark.parametrize("dt", ["f32", "bf16"])
 @pytest.mark.parametrize("K", [1, 2, 3, 4])
 def test_fused_many_buckets_per_cluster(K, dt, rule):
-    """Enough buckets that every cluster of the cluster kernel resolves a
-    dozen or more in turn (its pipelined hand-offs: the next bucket's Gram
-    streamed while the one before is solved), with ragged bucket sizes;
-    every bucket against the oracle."""
+    """Several buckets a streaming CTA and a dozen or more a solving team in turn
+    (the next bucket's Gram streamed while the one before is solved), with
+    ragged bucket sizes; every bucket against the oracle."""
     sizes = [7001 + 37 * i for i in range(260)]
     w = _workload(K, dt, sizes, 6000, seed=70 + K, flip=0.2)
     off, hv, out, beta, status, _ = _run(w, rule, dt, params=_fused_params(3, 4))
@@ -429,10 +427,9 @@ def test_fused_many_buckets_per_cluster(K, dt, rule):
 
 @pytest.mark.parametrize("K", [2, 4, 8])
 def test_fused_in_place_equals_out_of_place(K):
-    """In place (the direction written over the first gradient) the fused
-    kernels give the bit-identical result: every output position is read,
-    through its thread's own prefetch, by the thread that writes it, after
-    every Gram read of the bucket."""
+    """In place (the direction written over the first gradient) the one launch
+    gives the bit-identical result: every output position is read a second
+    time by the thread that writes it, after every Gram read of the bucket."""
     w = _workload(K, "bf16", RAGGED * 2, 180000, seed=30 + K)
     off, hv, out1, beta1, _, _ = _run(w, "mgda", "bf16", params=_fused_params())
     _, _, out2, beta2, _, _ = _run(w, "mgda", "bf16", params=_fused_params(), inplace=True)
@@ -441,13 +438,14 @@ def test_fused_in_place_equals_out_of_place(K):
 
 
 def test_per_plan_path_runs_the_fused_kernel_where_chosen():
-    """A plan for which bkmoo_resolve_path picks the cluster kernel (K = 4,
-    2 MiB fp32 buckets) resolves by it by default: the result is the one of
-    the forced fused path, bit for bit, and matches the oracle."""
+    """A plan for which bkmoo_resolve_launches says one (K = 4, 2 MiB fp32
+    buckets): the default result is that of the forced one launch, bit for
+    bit, and matches the oracle."""
     K = 4
     w = _workload(K, "f32", [3 * (1 << 19) + 12345], 1 << 19, seed=91)
     off = bk.bkmoo_plan(w.param_sizes, 4, w.bucket_bytes)
     assert bk.bkmoo_resolve_path(K, bk.BKMOO_F32, "mgda", off, 0) == 1
+    assert bk.bkmoo_resolve_launches(K, bk.BKMOO_F32, "mgda", off) == 1
     _, hv, out_auto, beta_auto, st, _ = _run(w, "mgda", "f32")
     _, _, out_f, beta_f, _, _ = _run(w, "mgda", "f32", params=_fused_params())
     np.testing.assert_array_equal(beta_auto, beta_f)
@@ -499,11 +497,11 @@ def test_fused_bounded_wait_reports_timeout():
 
 
 def test_cluster_bounded_exchange_wait_reports_timeout():
-    """Failure detection in the cluster kernel without a fault: CTA 0 of
-    every cluster withholds its first bucket's partial (a hand-off that
-    never comes), each peer's exchange wait ends after its bound and every
-    later wait at once, the call reports BKMOO_ERR_TIMEOUT, and the context
-    stays usable: the next resolve succeeds and matches the oracle."""
+    """Failure detection without a fault: CTA 0 withholds its first chunk's
+    partial (a hand-off that never comes), the solving team's wait for it ends
+    after its bound and every other wait at once, the call reports
+    BKMOO_ERR_TIMEOUT, and the context stays usable: the next resolve succeeds
+    and matches the oracle."""
     import time
     K = 4
     sizes = [7001 + 37 * i for i in range(260)]
