@@ -132,8 +132,8 @@ struct StreamShape {
 };
 StreamShape stream_shape(const PlanView& v, int rule, int sms) {
   // From a bucket's last partial to its coefficients on every SM (us), from
-  // globaltimer stamps under load (K = 2, 4, 8) and, for K <= 4, the lead at
-  // which 1 and 4 MiB buckets run fastest.
+  // globaltimer stamps under load (K = 2, 4, 8; K = 5..7 lie on the line between)
+  // and, for K <= 4, the lead at which 1 and 4 MiB buckets run fastest.
   const double k4 = v.K < 4 ? v.K : 4, more = v.K > 4 ? v.K - 4 : 0;
   const double chain = rule == BKMOO_CAGRAD   ? 8 + 2 * k4 + 6 * more
                        : rule == BKMOO_PCGRAD ? 1 + 2.25 * k4 + 9 * more
@@ -326,25 +326,22 @@ int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool 
   const bool pf = v.K >= gram_prefetch_min_k();
   const void* fn = pf ? gram_prefetch_fn(v.K, v.in_dtype) : gram_fn(v.K, v.in_dtype);
   int smem = pf ? gram_prefetch_smem(v.K) : 0, threads = kThreads, grid = 0;
+  // Fed by bulk copies: with at most a chunk per SM, where a register kernel's
+  // CTA has too little in flight alone (64 chunks, K = 2..8: 1.04-1.3 times as
+  // fast), and for K = 6 and 7, whose register kernels lose occupancy (3.2 GB: K =
+  // 6 bf16 512 -> 464 us, K = 7 fp32 481 -> 448; K = 2..5 and 8 within 3 % either
+  // way).  Not for one or two chunks, which gain nothing from the ring but wait
+  // for it to be set up (three launches, register / bulk: K = 8 fp32 one chunk
+  // 29.0 / 31.2 us, K = 6 bf16 two 25.4 / 27.2, three 30.3 / 29.2).
+  int sms = 0;
+  if (sm_count(&sms) != cudaSuccess) return BKMOO_ERR_CUDA;
   const void* bulk = gram_bulk_fn(v.K, v.in_dtype);
-  if (bulk) {
-    // Fed by bulk copies: with at most a chunk per SM, where a register
-    // kernel's CTA has too little in flight alone (64 chunks, K = 2..8: 1.04-1.3
-    // times as fast), and for K = 6 and 7, whose register kernels lose
-    // occupancy (3.2 GB: K = 6 bf16 512 -> 464 us, K = 7 fp32 481 -> 448; K = 2..5
-    // and 8 within 3 % either way).
-    int two = 0;   // two CTAs per SM
-    if (persistent_grid(bulk, gram_bulk_threads(), &two, gram_bulk_smem(v.K)) != cudaSuccess)
-      return BKMOO_ERR_CUDA;
-    if (2 * nch <= two || v.K == 6 || v.K == 7) {
-      fn = bulk;
-      smem = gram_bulk_smem(v.K);
-      threads = gram_bulk_threads();
-      grid = two;
-    }
+  if (bulk && nch > 2 && (nch <= sms || v.K == 6 || v.K == 7)) {
+    fn = bulk;
+    smem = gram_bulk_smem(v.K);
+    threads = gram_bulk_threads();
   }
-  if (fn != bulk && persistent_grid(fn, threads, &grid, smem) != cudaSuccess)
-    return BKMOO_ERR_CUDA;
+  if (persistent_grid(fn, threads, &grid, smem) != cudaSuccess) return BKMOO_ERR_CUDA;
   if (grid > nch) grid = (int)nch;
   GradPtrs ga = g;
   PlanView va = v;

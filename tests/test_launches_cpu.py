@@ -82,6 +82,10 @@ def test_cooperative_launch_that_does_not_fit_falls_back(fake):
     (3, BF16, PLAN * 2, ["gram", "solve", "combine-last-first"]),
     (8, F32, PLAN, ["gram", "solve", "combine-prefetch"]),
     (6, F32, PLAN, ["gram-bulk", "solve", "combine-prefetch"]),
+    (6, F32, [0, 5, 90], ["gram", "solve", "combine-prefetch"]),
+    (6, F32, [0, 5, 90, 91], ["gram-bulk", "solve", "combine-prefetch"]),
+    (8, F32, [0, 2 * 16384], ["gram", "solve", "combine-prefetch"]),
+    (8, F32, [0, 2 * 16384 + 1], ["gram-bulk", "solve", "combine-prefetch"]),
     (12, F32, PLAN, ["gram-prefetch", "solve", "combine-prefetch"]),
     (4, F32, [0, 152 * 16384], ["gram-bulk", "solve", "combine-prefetch"]),
     (4, F32, [0, 153 * 16384], ["gram", "solve", "combine-last-first"]),
