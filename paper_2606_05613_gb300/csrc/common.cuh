@@ -258,7 +258,9 @@ __device__ __forceinline__ double set_sum(const double* row, int64_t rs, int64_t
 // sums in the same way -- the order in which the streamed kernel, whose sets
 // are summed by different warps of a team, arrives at them.
 __device__ __forceinline__ double sum_chunk_rows(const double* src, int64_t rs, int64_t n, int K) {
+  if (n == 1) return *src;              // (adding zeros changes no partial)
   if (K > kStreamMaxK) return sum_rows8(src, rs, n);
+  if (n <= kSetChunks) return set_sum(src, rs, n);
   double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
   for (int64_t c = 0; c < n; c += 8 * kSetChunks) {
 #pragma unroll

@@ -87,11 +87,57 @@ __device__ void reduce_bucket(const PlanView& v, int64_t b, double* G, int lane)
 
 // n rows (rs doubles apart) by a block of eight warps: warp w forms the
 // interleaved sum w of every entry (t8: [8][P] in shared memory); tree8_entry
-// adds them once the block has synchronised.  `sets`: the rows are chunk rows
-// of K <= kStreamMaxK (sum_chunk_rows), else flat (sum_rows8).
+// adds them once the block has synchronised.
 constexpr int kWideWarps = 8;
+// Flat rows (sum_rows8), E entries a lane: rows w, w + 8, ..., U of them in one
+// round trip.  A copy for each E, inlined: with the entries tested at run time, or
+// out of line, fewer loads are in flight (Gram call, two buckets of 400 chunks, K
+// = 12: 134 us tested, 135 out of line, 123 so; K = 16: 178, 194, 175).
+template <int E>
+__device__ __forceinline__ void sum_flat_wide(const double* src, int64_t rs, int64_t n, int P,
+                                              double* t8, int lane, int w) {
+  constexpr int U = E == 1 ? 16 : E == 2 ? 8 : 4;
+  int f[E];
+  double t[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    f[e] = min(lane + 32 * e, P - 1);
+    t[e] = 0.0;
+  }
+  int64_t c = w;
+  const double* p = src + w * rs;
+  const int64_t step = kWideWarps * rs;
+  for (; c + (U - 1) * kWideWarps < n; c += kWideWarps * U, p += U * step) {
+    double x[U][E];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[u][e] = p[u * step + f[e]];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e) t[e] += x[u][e];
+  }
+  if (c < n) {
+    double x[U][E];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e) x[u][e] = c + u * kWideWarps < n ? p[u * step + f[e]] : 0.0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        if (c + u * kWideWarps < n) t[e] += x[u][e];
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (lane + 32 * e < P) t8[w * P + lane + 32 * e] = t[e];
+}
+// `sets`: the rows are chunk rows of K <= kStreamMaxK (sum_chunk_rows).
 __device__ void sum_rows_wide(const double* src, int64_t rs, int64_t n, int P, bool sets,
                               double* t8, int lane, int w) {
+  static_assert(tri(kMaxK) <= 160, "five entries a lane");
   if (sets) {
     for (int p = lane; p < P; p += 32) {
       double t = 0.0;
@@ -101,28 +147,11 @@ __device__ void sum_rows_wide(const double* src, int64_t rs, int64_t n, int P, b
     }
     return;
   }
-  // rows w, w + 8, ...: four rows of up to five entries a lane in flight
-  constexpr int E = (tri(kMaxK) + 31) / 32, U = 4;
-  double t[E] = {0.0, 0.0, 0.0, 0.0, 0.0};
-  static_assert(E == 5, "entries per lane");
-  for (int64_t c = w; c < n; c += kWideWarps * U) {
-    double x[U][E];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        x[u][e] = (c + u * kWideWarps < n && lane + 32 * e < P)
-                      ? src[(c + u * kWideWarps) * rs + lane + 32 * e]
-                      : 0.0;
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int e = 0; e < E; ++e)
-        if (c + u * kWideWarps < n && 32 * e < P) t[e] += x[u][e];
-  }
-#pragma unroll
-  for (int e = 0; e < E; ++e)
-    if (lane + 32 * e < P) t8[w * P + lane + 32 * e] = t[e];
+  if (P <= 32) sum_flat_wide<1>(src, rs, n, P, t8, lane, w);
+  else if (P <= 64) sum_flat_wide<2>(src, rs, n, P, t8, lane, w);
+  else if (P <= 96) sum_flat_wide<3>(src, rs, n, P, t8, lane, w);
+  else if (P <= 128) sum_flat_wide<4>(src, rs, n, P, t8, lane, w);
+  else sum_flat_wide<5>(src, rs, n, P, t8, lane, w);
 }
 __device__ __forceinline__ double tree8_entry(const double* t8, int P, int p) {
   const double* t = t8 + p;

@@ -326,7 +326,7 @@ def test_huge_buckets_group_reduction(dt):
         _check_against_oracle(w, rule, off, hv, out, beta.cpu().numpy(), status.cpu().numpy(), dt)
 
 
-@pytest.mark.parametrize("K", [1, 4, 9, 16])
+@pytest.mark.parametrize("K", [1, 4, 9, 12, 14, 16])
 def test_group_sums_beside_many_small_buckets(K):
     """Buckets of more than 1024 chunks at the front, in the middle and at the
     end of 11,000 small ones (several look-over rounds of the pre-reduction's

@@ -269,7 +269,7 @@ def test_bulk_fed_gram_is_the_register_kernels(K, dt):
             assert bad is None or not torch.isfinite(got).all()
 
 
-@pytest.mark.parametrize("K", [2, 8, 12])
+@pytest.mark.parametrize("K", [2, 8, 10, 12, 15, 16])
 def test_solve_pass_at_the_edges_of_its_two_kernels(K):
     """Plans on both sides of the lines between a block and a warp per bucket
     (two buckets per SM; the longest bucket against the number of buckets),
