@@ -363,9 +363,8 @@ const void* combine_prefetch_fn_k9_16(int K, int dti, int dto);
 int combine_prefetch_smem(int K);
 
 // Combine kernels that take the last chunk first, for short windows,
-// signature (GradPtrs, PlanView, void* out), K <= combine_last_first_max_k;
-// combine_*.cu.
-constexpr int combine_last_first_max_k(int dti) { return dti == BKMOO_F32 ? 4 : 3; }
+// signature (GradPtrs, PlanView, void* out), for the K that last_first_bytes
+// (host.cu) gives a size, nullptr for others; combine_*.cu.
 const void* combine_fn_f32(int K, int dtype_out);
 const void* combine_fn_bf16(int K, int dtype_out);
 

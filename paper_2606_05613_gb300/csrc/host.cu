@@ -352,26 +352,35 @@ int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool 
   return BKMOO_OK;
 }
 
+// The most gradient bytes of a short window, which is combined last chunk first
+// (combine_impl.cuh), out of L2, of which a Gram pass just over leaves 50-60 MB; 0
+// where the prefetching kernel always is the faster one.  Three launches on
+// inputs not in L2 before, the prefetching kernel / this one (us).  Few gradients:
+// K = 2 fp32, 40 MB of gradients 39.6 / 36.6, 80 MB 56.0 / 54.8, 120 MB 74.9 / 74.4,
+// 390 MB 163.7 / 169.6; K = 3 bf16, 60 MB 47.3 / 44.7, 180 MB 92.7 / 92.3, fp32 290
+// MB 118.2 / 123.0; K = 4 fp32, 60 MB 45.6 / 42.6, 105 MB 60.4 / 60.3, 240 MB 115.9
+// / 113.9, 390 MB 147.4 / 148.6.  With more to a vector its loads in flight do not
+// keep up: K = 4 bf16, 40 MB 41.2 / 43.8, 80 MB 51.4 / 55.8; K = 5 bf16, 63 MB 46.9 /
+// 57.6; K = 8 fp32, 80 MB 54.9 / 66.8; K = 16 fp32, 160 MB 110 / 129; K = 11 bf16 and
+// K = 12 to 15 fp32 within 4 % either way.  Many bf16 gradients, for which the
+// other's slots leave one CTA to an SM: 1.04-1.10 times as fast from 120 to 400 MB,
+// 1.02-1.05 to 600, 1.02 at 840, 0.99 at 1200 (K = 16, 160 MB 138 / 127, 420 MB 225
+// / 217).  Fewer chunks than SMs: within 2 us either way, at K = 12 to 15 up to 8 %
+// slower.
+double last_first_bytes(int K, int dt) {
+  const double mib = 1024.0 * 1024.0;
+  if (K <= (dt == BKMOO_F32 ? 4 : 3)) return 192.0 * mib;
+  return dt == BKMOO_BF16 && K >= 12 ? 768.0 * mib : 0.0;
+}
+
 int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_dtype,
                    cudaStream_t s) {
   const int64_t nch = v.c_hi - v.c_lo;
   if (nch <= 0) return BKMOO_OK;
-  // A short window of few gradients: last chunk first, out of L2, of which a Gram
-  // pass just over leaves 50-60 MB.  Three launches on inputs not in L2 before,
-  // the prefetching kernel / this one (us): K = 2 fp32, 40 MB of gradients 39.6 /
-  // 36.6, 80 MB 56.0 / 54.8, 120 MB 74.9 / 74.4, 390 MB 163.7 / 169.6; K = 3 bf16,
-  // 60 MB 47.3 / 44.7, 180 MB 92.7 / 92.3, fp32 290 MB 118.2 / 123.0; K = 4 fp32, 60
-  // MB 45.6 / 42.6, 105 MB 60.4 / 60.3, 240 MB 115.9 / 113.9, 390 MB 147.4 / 148.6.
-  // With more gradients to a vector its loads in flight do not keep up: K = 4
-  // bf16, 40 MB 41.2 / 43.8, 80 MB 51.4 / 55.8; K = 5 bf16, 63 MB 46.9 / 57.6; K = 8
-  // fp32, 80 MB 54.9 / 66.8; K = 16 fp32, 105 MB 64.0 / 88.7.  Fewer chunks than
-  // SMs: within 2 us either way (K = 2 fp32, 40 chunks 23.2 / 25.0, 100 chunks 26.7
-  // / 26.6).
   const double bytes = (double)nch * v.chunk_elems * v.K * elem_bytes(v.in_dtype);
   int sms = 0;
   if (sm_count(&sms) != cudaSuccess) return BKMOO_ERR_CUDA;
-  const bool shortw = v.K <= combine_last_first_max_k(v.in_dtype) &&
-                      bytes <= 192.0 * 1024 * 1024 && nch > sms;
+  const bool shortw = nch > sms && bytes <= last_first_bytes(v.K, v.in_dtype);
   const void* fn = shortw ? combine_fn(v.K, v.in_dtype, out_dtype)
                           : combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
   const int smem = shortw ? 0 : combine_prefetch_smem(v.K);

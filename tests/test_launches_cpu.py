@@ -91,6 +91,12 @@ def test_cooperative_launch_that_does_not_fit_falls_back(fake):
     (4, F32, [0, 153 * 16384], ["gram", "solve", "combine-last-first"]),
     (4, F32, [0, 768 * 16384], ["gram", "solve", "combine-last-first"]),      # 192 MiB
     (4, F32, [0, 768 * 16384 + 1], ["gram", "solve", "combine-prefetch"]),
+    (12, BF16, [0, 152 * 32768], ["gram-prefetch", "solve", "combine-prefetch"]),
+    (12, BF16, [0, 153 * 32768], ["gram-prefetch", "solve", "combine-last-first"]),
+    (16, BF16, [0, 768 * 32768], ["gram-prefetch", "solve", "combine-last-first"]),   # 768 MiB
+    (16, BF16, [0, 768 * 32768 + 1], ["gram-prefetch", "solve", "combine-prefetch"]),
+    (11, BF16, [0, 153 * 32768], ["gram", "solve", "combine-prefetch"]),
+    (16, F32, [0, 153 * 16384], ["gram-prefetch", "solve", "combine-prefetch"]),
     (4, F32, [0, 1025 * 16384], ["gram", "groups", "solve", "combine-prefetch"]),
 ])
 def test_kernels_of_the_three_launches(fake, K, dt, off, kernels):

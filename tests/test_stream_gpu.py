@@ -311,3 +311,31 @@ def test_combination_kernels_at_the_edges_of_their_rule(K, dt):
             _same(_run(res, grads, "mgda", odt, bk.BKMOO_FLAG_THREE_PASS, inplace),
                   _run(res, grads, "mgda", odt, bk.BKMOO_FLAG_FUSED, inplace))
         assert res.status() == 0
+
+
+@pytest.mark.parametrize("K", [12, 13, 16])
+def test_combination_of_many_bf16_gradients_last_chunk_first(K):
+    """K >= 12 bf16, windows of one chunk more than SMs, and of as many (the
+    prefetching kernel): the direction is that of the weights, in place too."""
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+    ch = 32768
+    for n in (sms, sms + 1):
+        sizes = [ch + 9] * 3 + [(n - 8) * ch - 5] + [7, 2]
+        off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+        grads = _grads(K, BF16, int(off[-1]), n)
+        res = bk.Resolver(K, BF16, off, DEV)
+        got, w, st = _run(res, grads, "mgda", F32, 0)
+        half = _run(res, grads, "mgda", BF16, 0)[0]
+        place = _run(res, grads, "mgda", BF16, 0, inplace=True)[0]
+        assert res.status() == 0 and not st.any()
+        for b in range(len(sizes)):
+            lo, hi = int(off[b]), int(off[b + 1])
+            want = torch.zeros(hi - lo, dtype=torch.float64, device=DEV)
+            size = torch.zeros_like(want)
+            for k in range(K):
+                x = grads[k][lo:hi].double() * w[b, k].double()
+                want += x
+                size += x.abs()
+            # K fp32 multiply-adds in a row
+            assert ((got[lo:hi] - want).abs() <= K * 2.0 ** -24 * size).all()
+        assert torch.equal(half, got.to(BF16)) and torch.equal(place, half)
