@@ -175,13 +175,12 @@ cudaError_t launch_group_reduce(const PlanView& v, cudaStream_t s, bool behind) 
 // us for each row of the longest bucket against 0.02 for each bucket, where that
 // bucket is long (1000 buckets of 300 elements beside one of 1000 chunks, K = 4:
 // 169 against 182, 2000 beside one of 400 147 against 116).
-static cudaError_t solve_wide(const PlanView& v, int64_t nb, bool* wide) {
-  int sms = 0;
-  const cudaError_t e = sm_count(&sms);
+static cudaError_t solve_wide(const PlanView& v, int64_t nb, bool* wide, int* sms) {
+  const cudaError_t e = sm_count(sms);
   const int64_t rows = v.max_chunks > kGroupMinChunks
                            ? (v.max_chunks + kGroupChunks - 1) / kGroupChunks
                            : v.max_chunks;
-  *wide = nb <= 2 * (int64_t)sms || 2 * rows >= nb;
+  *wide = nb <= 2 * (int64_t)*sms || 2 * rows >= nb;
   return e;
 }
 
@@ -190,8 +189,15 @@ cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_wei
   const int64_t nb = v.b_hi - v.b_lo;
   if (nb <= 0) return cudaSuccess;
   bool wide = false;
-  const cudaError_t e = solve_wide(v, nb, &wide);
+  int sms = 0;
+  const cudaError_t e = solve_wide(v, nb, &wide, &sms);
   if (e != cudaSuccess) return e;
+  // A few us of solve on every SM: more than six buckets per SM by exact MGDA (1024
+  // buckets of 4099 elements, plain / behind: K = 4 52.6 / 47.1 us, K = 5 66.9 / 54.9;
+  // PCGrad 56.9 / 55.5 and 69.2 / 65.8, but K = 8 109.7 / 126.2, its MGDA 97.5 / 99.3,
+  // and K = 2 CAGrad 43.4 / 50.2; 608 buckets, MGDA, K = 4 28.7 / 30.0).
+  const bool many_short = p.rule == BKMOO_MGDA && (p.flags & BKMOO_FLAG_POLISH) && v.K < 8 &&
+                          nb > 6 * (int64_t)sms;
   const int64_t grid = wide ? nb : (nb + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
   PlanView va = v;
   SolveParams pa = p;
@@ -199,7 +205,7 @@ cudaError_t launch_solve(const PlanView& v, const SolveParams& p, float* out_wei
   return launch_behind(wide ? (const void*)solve_wide_kernel : (const void*)solve_kernel,
                        dim3((unsigned)grid),
                        dim3(32 * (wide ? kWideWarps : kSolveWarpsPerBlock)), args, 0, s,
-                       behind && wide);
+                       behind && (wide || many_short));
 }
 
 cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream_t s,
@@ -207,7 +213,8 @@ cudaError_t launch_gram_finalize(const PlanView& v, double* out_gram, cudaStream
   const int64_t nb = v.n_buckets;
   if (nb == 0) return cudaSuccess;
   bool wide = false;
-  const cudaError_t e = solve_wide(v, nb, &wide);
+  int sms = 0;
+  const cudaError_t e = solve_wide(v, nb, &wide, &sms);
   if (e != cudaSuccess) return e;
   const int64_t grid = wide ? nb : (nb + kSolveWarpsPerBlock - 1) / kSolveWarpsPerBlock;
   PlanView va = v;
