@@ -139,6 +139,7 @@ struct PlanView {
   // [b_lo, b_hi) (the whole plan except in the windowed host-memory path).
   int64_t c_lo, c_hi;
   int64_t b_lo, b_hi;
+  int64_t elems;        // elements of one language in [b_lo, b_hi) (host-computed)
   int64_t max_chunks;   // most chunks in one bucket of the plan (host-computed)
 };
 

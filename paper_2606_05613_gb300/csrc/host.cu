@@ -113,10 +113,10 @@ const void* stream_fn(int K, int dt) {
 //    of 65.5 GB 20.66 / 20.61; K = 3 1.2 GiB 3.91 / 3.87; K = 5 1 GiB 2.47 / 2.46; K = 8
 //    0.8 GiB 1.89 / 1.92, one of 20 GB 6.15 / 5.92); K <= 2, whose second read costs
 //    less, from 32 GiB (K = 2 4 GB 2.81 / 2.90; K = 1 the same within 1 %).
-bool stream_wins(const PlanView& v, const int64_t* off) {
+bool stream_wins(const PlanView& v) {
   if (v.K > kStreamMaxK || v.c_hi <= v.c_lo) return false;
   const int64_t nb = v.b_hi - v.b_lo;
-  const double bytes = (double)(off[v.b_hi] - off[v.b_lo]) * v.K * elem_bytes(v.in_dtype);
+  const double bytes = (double)v.elems * v.K * elem_bytes(v.in_dtype);
   const double mib = 1024.0 * 1024.0;
   if (v.K >= 5)
     return bytes >= 96.0 * mib && bytes >= 1.0 * mib * nb &&
@@ -241,11 +241,10 @@ bool solve_is_short(int32_t K, int32_t rule, const bkmoo_params& p) {
 
 // Whether a resolve of the view's window takes the streamed launch: the one
 // rule behind bkmoo_resolve, bkmoo_resolve_buckets and bkmoo_resolve_launches.
-bool streams(const PlanView& v, const int64_t* off, int32_t rule, const bkmoo_params& p,
-             uint32_t flags) {
+bool streams(const PlanView& v, int32_t rule, const bkmoo_params& p, uint32_t flags) {
   if ((flags & BKMOO_FLAG_THREE_PASS) || !solve_is_short(v.K, rule, p)) return false;
   if (flags & BKMOO_FLAG_FUSED) return v.K <= kStreamMaxK && v.c_hi > v.c_lo;
-  return stream_wins(v, off);
+  return stream_wins(v);
 }
 
 // bkmoo_resolve_path's answer (see bkmoo.h); decides nothing.
@@ -281,6 +280,7 @@ void plan_sizes(int32_t K, int32_t dt, const int64_t* offsets, int64_t B, PlanVi
   v->n_buckets = B;
   v->n_chunks = count_chunks(offsets, B, ch);
   v->chunk_elems = ch;
+  v->elems = offsets[B];
   v->max_chunks = 0;
   for (int64_t b = 0; b < B; ++b) {
     const int64_t n = (offsets[b + 1] - offsets[b] + ch - 1) / ch;
@@ -377,7 +377,7 @@ int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_
                    cudaStream_t s) {
   const int64_t nch = v.c_hi - v.c_lo;
   if (nch <= 0) return BKMOO_OK;
-  const double bytes = (double)nch * v.chunk_elems * v.K * elem_bytes(v.in_dtype);
+  const double bytes = (double)v.elems * v.K * elem_bytes(v.in_dtype);
   int sms = 0;
   if (sm_count(&sms) != cudaSuccess) return BKMOO_ERR_CUDA;
   const bool shortw = nch > sms && bytes <= last_first_bytes(v.K, v.in_dtype);
@@ -614,7 +614,7 @@ int bkmoo_resolve(const void* const* grads, int32_t K, int32_t in_dtype, const i
   cudaEvent_t* ev = static_cast<cudaEvent_t*>(prm.events);
   const SolveParams sp = solve_params(rule, prm, prm.flags);
   if (ev && cudaEventRecord(ev[0], s) != cudaSuccess) return BKMOO_ERR_CUDA;
-  if (streams(v, offsets, rule, prm, prm.flags)) {
+  if (streams(v, rule, prm, prm.flags)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, true, &taken, s);
     if (r != BKMOO_OK) return r;
@@ -655,6 +655,7 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   v.c_lo = c;
   for (int64_t b = b_lo; b < b_hi; ++b) c += (offsets[b + 1] - offsets[b] + v.chunk_elems - 1) / v.chunk_elems;
   v.c_hi = c;
+  v.elems = offsets[b_hi] - offsets[b_lo];
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const uint32_t flags = prm.flags & ~BKMOO_FLAG_FUSED;
   const SolveParams sp = solve_params(rule, prm, flags);
@@ -662,7 +663,7 @@ int bkmoo_resolve_buckets(const void* const* grads, int32_t K, int32_t in_dtype,
   // the caller overlaps them with; the streamed launch needs all of them at
   // once (a training step that resolves each bucket beside the backward pass:
   // 263.9 ms with three launches per bucket, 267.3 streamed).
-  if (b_hi - b_lo > 2 && streams(v, offsets, rule, prm, flags)) {
+  if (b_hi - b_lo > 2 && streams(v, rule, prm, flags)) {
     bool taken = false;
     r = launch_stream(g, v, sp, ws, out_weights, out_status, out_dir, out_dtype, false, &taken, s);
     if (r != BKMOO_OK || taken) return r;
@@ -778,6 +779,7 @@ int bkmoo_resolve_host(const void* const* host_grads, int32_t K, int32_t in_dtyp
     PlanView vw = v;
     vw.b_lo = b0;
     vw.b_hi = b1;
+    vw.elems = n;
     // chunk range of the window: chunks are numbered bucket by bucket
     vw.c_lo = c_next;
     for (int64_t b = b0; b < b1; ++b) c_next += (offsets[b + 1] - offsets[b] + ch - 1) / ch;
@@ -864,7 +866,7 @@ int bkmoo_resolve_launches(int32_t K, int32_t in_dtype, int32_t rule, const int6
   std::memset(&v, 0, sizeof v);
   plan_sizes(K, in_dtype, offsets, n_buckets, &v);
   if (n_buckets == 0) *launches = 0;
-  else if (streams(v, offsets, rule, prm, prm.flags)) *launches = 1;
+  else if (streams(v, rule, prm, prm.flags)) *launches = 1;
   else *launches = v.max_chunks > kGroupMinChunks ? 4 : 3;
   return BKMOO_OK;
 }

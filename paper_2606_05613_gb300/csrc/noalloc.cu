@@ -160,6 +160,7 @@ extern "C" int bkmoo_gram_noalloc(const void* const* grads, int32_t K, int32_t i
   v.plan_hash = t.hdr.plan_hash;
   v.K = K;
   v.in_dtype = in_dtype;
+  v.elems = offsets[n_buckets];
   v.max_chunks = 0;
   for (int64_t b = 0; b < n_buckets; ++b) {
     const int64_t nb = (offsets[b + 1] - offsets[b] + ch - 1) / ch;
