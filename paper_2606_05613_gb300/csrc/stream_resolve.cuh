@@ -15,7 +15,7 @@
 // MB: a probe that re-reads a stream D bytes later finds all of it up to D = 60
 // MB with evict_last, 45 MB of it at D = 120 MB), so a shorter chain means fewer
 // bytes.  Three launches against this one (us): GPT-2 small 672, 520; 250 M fp32
-// elements K = 4 in 1 MiB buckets 1279, 820; 500 M K = 2 in 4 MiB buckets 1470, 874.
+// elements K = 4 in 1 MiB buckets 1279, 820; 500 M K = 2 in 4 MiB buckets 1496, 882.
 //
 // Chunks and arithmetic are those of the three launches: the same chunks, the
 // same thread for every vector, the same order of every sum, so the results
