@@ -15,9 +15,9 @@
 // else, so in-place use is race-free.
 //
 // This kernel takes the last chunk first, for windows of a few chunks per CTA:
-// what the Gram pass read last is then still in L2 (up to about 60 MB of it).
-// Long windows, of which L2 holds little, take combine_prefetch_kernel, whose
-// copies in flight move 2-6 % more per second.
+// what the Gram pass read last is then still in L2 (up to about 60 MB of it); and
+// it serves short chunks, which end before combine_prefetch_kernel's copies are in
+// flight.  Other windows take that kernel, which moves 2-6 % more per second.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -83,9 +83,9 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const GradPtrs g, con
     const int nv = (int)((ve - vs) / EPV);
 
     int i = threadIdx.x;
-    // K >= 12: two vectors per thread in flight (8 % faster at K = 16; no change at
+    // K >= 9: two vectors per thread in flight (8 % faster at K = 16; no change at
     // K = 4 and 8, where the occupancy already hides the latency)
-    if (K >= 12) {
+    if (K >= 9) {
       for (; i + kThreads < nv; i += 2 * kThreads) {
         const int64_t el0 = vs + (int64_t)i * EPV, el1 = el0 + (int64_t)kThreads * EPV;
         uint4 r0[K], r1[K];
@@ -139,5 +139,14 @@ __global__ void __launch_bounds__(kThreads) combine_kernel(const GradPtrs g, con
 #define BKMOO_COMBINE_ROW(K, DTI)                                        \
   {(const void*)combine_kernel<K, DTI, BKMOO_F32>,                       \
    (const void*)combine_kernel<K, DTI, BKMOO_BF16>}
+
+#define BKMOO_COMBINE_TABLE(DTI)                                                          \
+  static const void* const kCombineTable[kMaxK][2] = {                                    \
+      BKMOO_COMBINE_ROW(1, DTI),  BKMOO_COMBINE_ROW(2, DTI),  BKMOO_COMBINE_ROW(3, DTI),  \
+      BKMOO_COMBINE_ROW(4, DTI),  BKMOO_COMBINE_ROW(5, DTI),  BKMOO_COMBINE_ROW(6, DTI),  \
+      BKMOO_COMBINE_ROW(7, DTI),  BKMOO_COMBINE_ROW(8, DTI),  BKMOO_COMBINE_ROW(9, DTI),  \
+      BKMOO_COMBINE_ROW(10, DTI), BKMOO_COMBINE_ROW(11, DTI), BKMOO_COMBINE_ROW(12, DTI), \
+      BKMOO_COMBINE_ROW(13, DTI), BKMOO_COMBINE_ROW(14, DTI), BKMOO_COMBINE_ROW(15, DTI), \
+      BKMOO_COMBINE_ROW(16, DTI)}
 
 }  // namespace bkmoo

@@ -363,9 +363,9 @@ const void* combine_prefetch_fn(int K, int dti, int dto);
 const void* combine_prefetch_fn_k9_16(int K, int dti, int dto);
 int combine_prefetch_smem(int K);
 
-// Combine kernels that take the last chunk first, for short windows,
-// signature (GradPtrs, PlanView, void* out), for the K that last_first_bytes
-// (host.cu) gives a size, nullptr for others; combine_*.cu.
+// Combine kernels that take the last chunk first, for short windows and short
+// chunks (last_first_bytes in host.cu), signature (GradPtrs, PlanView, void* out);
+// combine_*.cu.
 const void* combine_fn_f32(int K, int dtype_out);
 const void* combine_fn_bf16(int K, int dtype_out);
 

@@ -366,9 +366,15 @@ int launch_gram_pass(const GradPtrs& g, const PlanView& v, cudaStream_t s, bool 
 // other's slots leave one CTA to an SM: 1.04-1.10 times as fast from 120 to 400 MB,
 // 1.02-1.05 to 600, 1.02 at 840, 0.99 at 1200 (K = 16, 160 MB 138 / 127, 420 MB 225
 // / 217).  Fewer chunks than SMs: within 2 us either way, at K = 12 to 15 up to 8 %
-// slower.
-double last_first_bytes(int K, int dt) {
+// slower.  Chunks little more than half full on average at most, every K, as far
+// as measured: 1024 buckets of a sixteenth, an eighth and a half of a chunk K = 5 fp32
+// 1.14, 1.15 and 1.08 times as fast, K = 8 fp32 1.18, 1.19, 1.02, K = 16 bf16 1.07,
+// 1.08, 1.06; 3000 of an eighth and a half K = 4 bf16 1.18, 1.02, K = 7 bf16 1.23,
+// 0.97, K = 12 fp32 (1.2 GB) 1.25, 1.02; 1024 of one chunk and 3 elements K = 3 fp32
+// 1.12; of whole ones 0.95-1.03.
+double last_first_bytes(int K, int dt, bool short_chunks) {
   const double mib = 1024.0 * 1024.0;
+  if (short_chunks) return 1024.0 * mib;
   if (K <= (dt == BKMOO_F32 ? 4 : 3)) return 192.0 * mib;
   return dt == BKMOO_BF16 && K >= 12 ? 768.0 * mib : 0.0;
 }
@@ -380,7 +386,8 @@ int launch_combine(const GradPtrs& g, const PlanView& v, void* out, int32_t out_
   const double bytes = (double)v.elems * v.K * elem_bytes(v.in_dtype);
   int sms = 0;
   if (sm_count(&sms) != cudaSuccess) return BKMOO_ERR_CUDA;
-  const bool shortw = nch > sms && bytes <= last_first_bytes(v.K, v.in_dtype);
+  const bool shortw = nch > sms && bytes <= last_first_bytes(v.K, v.in_dtype,
+                                                             16 * v.elems <= 9 * nch * v.chunk_elems);
   const void* fn = shortw ? combine_fn(v.K, v.in_dtype, out_dtype)
                           : combine_prefetch_fn(v.K, v.in_dtype, out_dtype);
   const int smem = shortw ? 0 : combine_prefetch_smem(v.K);

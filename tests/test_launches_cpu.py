@@ -91,6 +91,13 @@ def test_cooperative_launch_that_does_not_fit_falls_back(fake):
     (4, F32, [0, 153 * 16384], ["gram", "solve", "combine-last-first"]),
     (4, F32, [0, 768 * 16384], ["gram", "solve", "combine-last-first"]),      # 192 MiB
     (4, F32, [0, 768 * 16384 + 1], ["gram", "solve", "combine-prefetch"]),
+    # 200 chunks, nine sixteenths full and a little more
+    (8, F32, np.arange(0, 201) * 9216, ["gram", "solve", "combine-last-first"]),
+    (8, F32, np.arange(0, 201) * 9217, ["gram", "solve", "combine-prefetch"]),
+    (8, F32, np.arange(0, 153) * 9216, ["gram-bulk", "solve", "combine-prefetch"]),
+    # 1 GiB of half-full chunks
+    (8, F32, np.arange(0, 4097) * 8192, ["gram", "solve", "combine-last-first"]),
+    (8, F32, np.arange(0, 4098) * 8192, ["gram", "solve", "combine-prefetch"]),
     # 1001 chunks of a quarter of their length: 66 MB
     (4, F32, np.arange(0, 1002) * 4097, ["gram", "solve", "combine-last-first"]),
     (12, BF16, [0, 152 * 32768], ["gram-prefetch", "solve", "combine-prefetch"]),

@@ -313,21 +313,24 @@ def test_combination_kernels_at_the_edges_of_their_rule(K, dt):
         assert res.status() == 0
 
 
-@pytest.mark.parametrize("K", [12, 13, 16])
-def test_combination_of_many_bf16_gradients_last_chunk_first(K):
-    """K >= 12 bf16, windows of one chunk more than SMs, and of as many (the
-    prefetching kernel): the direction is that of the weights, in place too."""
+@pytest.mark.parametrize("dt", [F32, BF16])
+@pytest.mark.parametrize("K", [5, 8, 9, 12, 13, 16])
+def test_combination_of_many_gradients_last_chunk_first(K, dt):
+    """Windows of one chunk more than SMs, and of as many (K >= 12 bf16 changes
+    kernels), and of short chunks (every K): the direction is that of the
+    weights, in place too."""
     sms = torch.cuda.get_device_properties(DEV).multi_processor_count
-    ch = 32768
-    for n in (sms, sms + 1):
-        sizes = [ch + 9] * 3 + [(n - 8) * ch - 5] + [7, 2]
+    ch = 16384 if dt == F32 else 32768
+    for sizes in ([ch + 9] * 3 + [(sms - 8) * ch - 5] + [7, 2],
+                  [ch + 9] * 3 + [(sms - 7) * ch - 5] + [7, 2],
+                  [ch // 2 - 3, 5, ch // 4 + 1] * 40 + [4097] * sms):
         off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
-        grads = _grads(K, BF16, int(off[-1]), n)
-        res = bk.Resolver(K, BF16, off, DEV)
-        got, w, st = _run(res, grads, "mgda", F32, 0)
+        grads = _grads(K, dt, int(off[-1]), K)
+        res = bk.Resolver(K, dt, off, DEV)
+        got, w, _ = _run(res, grads, "mgda", F32, 0)   # (2 elements: a singular Gram)
         half = _run(res, grads, "mgda", BF16, 0)[0]
-        place = _run(res, grads, "mgda", BF16, 0, inplace=True)[0]
-        assert res.status() == 0 and not st.any()
+        place = _run(res, grads, "mgda", dt, 0, inplace=True)[0]
+        assert res.status() == 0
         for b in range(len(sizes)):
             lo, hi = int(off[b]), int(off[b + 1])
             want = torch.zeros(hi - lo, dtype=torch.float64, device=DEV)
@@ -338,4 +341,4 @@ def test_combination_of_many_bf16_gradients_last_chunk_first(K):
                 size += x.abs()
             # K fp32 multiply-adds in a row
             assert ((got[lo:hi] - want).abs() <= K * 2.0 ** -24 * size).all()
-        assert torch.equal(half, got.to(BF16)) and torch.equal(place, half)
+        assert torch.equal(half, got.to(BF16)) and torch.equal(place, got.to(dt))
